@@ -42,6 +42,7 @@ namespace {
 
 constexpr uint64_t kPlanMagic = 0x5241444f4e504c4eULL;   // "RADONPLN"
 constexpr int kPlanThreads = 256;
+constexpr int kAdjThreads = 128;     // adjoint: each thread owns a vertical pair of a 16 x 16 tile's pixels
 constexpr int kMaxChunkViews = 32;   // adjoint: views per staged chunk at most (16 where 32 do not fit)
 
 struct Unit {
@@ -266,26 +267,39 @@ __global__ void __launch_bounds__(kPlanThreads) single_forward_kernel(const Unit
 
 // ------------------------------------------------------------------------------------- adjoint
 
+// One view of a parallel-beam chunk, as the gather of a tile reads it (tile-local pixel p):
+//   t' = ax px + ay py + a0   window-relative detector coordinate, shifted so that its nearest integer is
+//                             the first candidate ray (for the counted gather; unshifted for the loop)
+//   s' = bx px + by py + c    the same along the rays: its nearest integer is the first candidate sample
+//   (Ax, Ay), (sx, sy), (nx, ny)   window ray 0's reference sample relative to the tile, the step along a
+//                             ray and the offset from one ray's samples to the next ray's
+struct alignas(16) AdjView {
+    float ax, ay, a0, c;
+    float Ax, Ay, sx, sy;
+    float nx, ny, bx, by;
+};
+
 struct AdjShared {
-    ViewF view[kMaxChunkViews];
+    union {
+        AdjView par[kMaxChunkViews];   // parallel beam
+        ViewF view[kMaxChunkViews];    // fan beam
+    };
     int dlo[kMaxChunkViews];
     float r[kMaxChunkViews];
-    // parallel beams: the window's first ray's sample nearest the tile centre (tile-relative) and
-    // step, the offset between neighbouring rays' samples of one lattice index, and the window
-    // constants (step / h^2, C) of the candidate samples
-    float4 ref[kMaxChunkViews];
-    float4 bc[kMaxChunkViews];   // (bx, by, C, -)
-    float2 dn[kMaxChunkViews];
     int w;
 };
 
 // Staging buffers of the adjoint's view chunks in dynamic shared memory.
 struct AdjBuffers {
     AdjShared* sh;
-    float4* rp;   // [chunk * wd] re-based ray positions and steps
+    float4* rp;   // [chunk * wd] re-based ray positions and steps (fan beam)
     float* ys;    // [chunk * wd] sinogram values
-    float* rc;    // [chunk * wd] window constants
+    float* rc;    // [chunk * wd] window constants (fan beam)
 };
+
+// Rays of a staged parallel-beam window beyond the detector window, holding zeros: the counted gather
+// steps through its rays without clamping the first one into the window.
+constexpr int kAdjPad = 2;
 
 // `cap` views per chunk at most, `max_wd` rays per view window.
 __device__ __forceinline__ AdjBuffers adj_buffers(unsigned char* smem_raw, int max_wd, int cap) {
@@ -297,26 +311,30 @@ __device__ __forceinline__ AdjBuffers adj_buffers(unsigned char* smem_raw, int m
     return b;
 }
 
+// Tile-local pixels of thread `tid`: (pi, pj) and the one below it.  Each warp takes an 8 x 8 block, each
+// group of eight lanes (one 16-byte shared-load phase) a 4 x 4 block.
+__device__ __forceinline__ void adj_pair_of(int tid, int* pi, int* pj) {
+    const int warp = tid >> 5, lane = tid & 31;
+    const int grp = lane >> 3, e8 = lane & 7;
+    *pi = (warp >> 1) * 8 + ((grp >> 1) * 2 + (e8 >> 2)) * 2;
+    *pj = (warp & 1) * 8 + (grp & 1) * 4 + (e8 & 3);
+}
+
 // Work item `tile` of unit u (a 16 x 16 pixel tile over all views), stored through the epilogue
-// (the identity for plans).  Every thread of the CTA calls it (it holds CTA barriers).  FAN = u.fan:
-// a parallel-beam view's detector coordinate is affine in the pixel (denominator 1), so its division
-// is left out (the same bits: the approximate quotient by 1 is exact).
-template <typename T, int KW, bool FAN>
+// (the identity for plans).  Every thread of the CTA calls it (it holds CTA barriers).  Fan beams.
+template <typename T, int KW>
 __device__ void plan_adjoint_tile(const Unit& u, int tile, const AdjBuffers& b, const Epilogue& ep, int* err) {
     const int tid = threadIdx.x;
-    const int warp = tid >> 5, lane = tid & 31;
-    // 4 x 8 pixels per warp, each group of eight lanes (one 16-byte shared-load phase) a 4 x 2 block
-    const int pi = (warp >> 1) * 4 + ((lane & 7) >> 1), pj = (warp & 1) * 8 + (lane >> 3) * 2 + (lane & 1);
-    const f32x2 p2 = f2_pack((float)pj, (float)pi);
+    int pi0, pj;
+    adj_pair_of(tid, &pi0, &pj);
     const int tiles_x = (u.n + kBwdTile - 1) / kBwdTile;
     const int ti = (tile / tiles_x) * kBwdTile, tj = (tile - (tile / tiles_x) * tiles_x) * kBwdTile;
-    const float gx = (float)(tj + pj), gy = (float)(ti + pi);
-    const bool inside = (ti + pi) < u.n && (tj + pj) < u.n;
+    const float gx = (float)(tj + pj);
     const f32x2 ih2_2 = f2_pack(u.ih2, u.ih2);
     const T* y = static_cast<const T*>(u.in);
     const int CV = u.cfg, wd = u.wd;
-    float acc = 0.0f;
-    bool viol = false;
+    float acc[2] = {0.0f, 0.0f};
+    bool viol[2] = {false, false};
     for (int c0 = 0; c0 < u.V; c0 += CV) {
         const int nv = min(CV, u.V - c0);
         if (tid < nv) {
@@ -329,7 +347,7 @@ __device__ void plan_adjoint_tile(const Unit& u, int tile, const AdjBuffers& b, 
             b.sh->r[tid] = r;
         }
         __syncthreads();
-        for (int e = tid; e < nv * wd; e += kPlanThreads) {
+        for (int e = tid; e < nv * wd; e += kAdjThreads) {
             const int vl = e / wd, dl = e - (e / wd) * wd;
             const int d = b.sh->dlo[vl] + dl;
             const bool valid = d >= 0 && d < u.D;
@@ -345,27 +363,34 @@ __device__ void plan_adjoint_tile(const Unit& u, int tile, const AdjBuffers& b, 
             const ViewF vf = b.sh->view[vl];
             const int dlo = b.sh->dlo[vl];
             const float r = b.sh->r[vl];
-            const float num = fmaf(vf.ax, gx, fmaf(vf.ay, gy, vf.a0));
-            const float t = FAN ? __fdividef(num, fmaf(vf.bx, gx, fmaf(vf.by, gy, vf.b0))) : num;
-            const float flo = ceilf(t - r), fhi = floorf(t + r);
-            const int da = (int)fmaxf(flo, (float)max(dlo, 0));
-            const int db = (int)fminf(fhi, (float)min(u.D - 1, dlo + wd - 1));
-            // a window that misses a candidate is reported once per pixel, after the views
-            viol |= (flo < (float)dlo && flo >= 0.0f) || (fhi > (float)(dlo + wd - 1) && fhi <= (float)(u.D - 1));
             const ulonglong2* rpv = reinterpret_cast<const ulonglong2*>(b.rp) + vl * wd;
             const float* yv = b.ys + vl * wd;
             const float* cv = b.rc + vl * wd;
-            for (int d = da; d <= db; ++d) {
-                const ulonglong2 rr = rpv[d - dlo];
-                acc = fmaf(bwd_ray_weight_c<KW>(p2, (float)pj, (float)pi, rr.x, rr.y, ih2_2, cv[d - dlo]), yv[d - dlo], acc);
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                const float px = (float)pj, py = (float)(pi0 + x), gy = (float)(ti + pi0 + x);
+                const f32x2 p2 = f2_pack(px, py);
+                const float num = fmaf(vf.ax, gx, fmaf(vf.ay, gy, vf.a0));
+                const float t = __fdividef(num, fmaf(vf.bx, gx, fmaf(vf.by, gy, vf.b0)));
+                const float flo = ceilf(t - r), fhi = floorf(t + r);
+                const int da = (int)fmaxf(flo, (float)max(dlo, 0));
+                const int db = (int)fminf(fhi, (float)min(u.D - 1, dlo + wd - 1));
+                // a window that misses a candidate is reported once per pixel, after the views
+                viol[x] |= (flo < (float)dlo && flo >= 0.0f) || (fhi > (float)(dlo + wd - 1) && fhi <= (float)(u.D - 1));
+                for (int d = da; d <= db; ++d) {
+                    const ulonglong2 rr = rpv[d - dlo];
+                    acc[x] = fmaf(bwd_ray_weight_c<KW>(p2, px, py, rr.x, rr.y, ih2_2, cv[d - dlo]), yv[d - dlo], acc[x]);
+                }
             }
         }
         __syncthreads();
     }
-    if (inside && viol) record_device_error(err, RADON_ERR_DEVICE_BOUNDS);
-    if (inside) {
-        const long long idx = (long long)(ti + pi) * u.n + (tj + pj);
-        static_cast<T*>(u.out)[idx] = from_f32<T>(epilogue_value<T>(ep, u.h * acc, idx));
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        if ((ti + pi0 + x) >= u.n || (tj + pj) >= u.n) continue;
+        if (viol[x]) record_device_error(err, RADON_ERR_DEVICE_BOUNDS);
+        const long long idx = (long long)(ti + pi0 + x) * u.n + (tj + pj);
+        static_cast<T*>(u.out)[idx] = from_f32<T>(epilogue_value<T>(ep, u.h * acc[x], idx));
     }
 }
 
@@ -376,122 +401,159 @@ __device__ void plan_adjoint_tile(const Unit& u, int tile, const AdjBuffers& b, 
 // per view (the same lattice index on every ray) and steps from one candidate ray to the next by
 // det_spacing * n.  Every lattice point within a pixel's 2 x 2 support lies inside the support box,
 // so it is a sample of its ray whenever the ray exists; rays outside the detector have zero values.
-// NC > 0: every candidate window [t - r, t + r] is shorter than NC rays and the staged window holds
-// at least NC, so each pixel steps through exactly NC rays from its first candidate (moved back
-// inside the window at its end), unrolled; rays beyond the pixel's support square carry weight zero
-// and add nothing.  NC = 0: a loop over the pixel's candidates.
+// NC > 0: every candidate window [t - r, t + r] is shorter than NC rays, so each pixel steps through
+// exactly NC rays from its first candidate, unrolled; rays beyond the pixel's support square carry
+// weight zero and add nothing (past the staged window lie kAdjPad zero values).  NC = 0: a loop over
+// the pixel's candidates.
+// Bound by issue: per pixel and view NC x KW samples of ~4 instructions each, plus the view's set-up.  So
+// a thread owns a vertical pair of pixels: one read of the view's record and one address base serve
+// both, the second pixel's coordinates are one addition away, the nearest-integer of a coordinate shifted
+// by 1/2 (adding and subtracting 1.5 * 2^23) takes the place of the conversions and clamps, and
+// eight CTAs of 128 threads hold a whole 512^2 image in one wave.
 template <typename T, int KW, int NC>
 __device__ void plan_adjoint_tile_parallel(const Unit& u, int tile, const AdjBuffers& b, const Epilogue& ep,
                                            int* err) {
+    constexpr float kMagic = 12582912.0f;        // 1.5 * 2^23: x + kMagic rounds x to the nearest integer
+    constexpr unsigned kMagicBits = 0x4B400000u;
     const int tid = threadIdx.x;
-    const int warp = tid >> 5, lane = tid & 31;
-    // 4 x 8 pixels per warp, each group of eight lanes (one shared-load phase) a 4 x 2 block
-    const int pi = (warp >> 1) * 4 + ((lane & 7) >> 1), pj = (warp & 1) * 8 + (lane >> 3) * 2 + (lane & 1);
-    const float px = (float)pj, py = (float)pi;
+    int pi0, pj;
+    adj_pair_of(tid, &pi0, &pj);
     const int tiles_x = (u.n + kBwdTile - 1) / kBwdTile;
     const int ti = (tile / tiles_x) * kBwdTile, tj = (tile - (tile / tiles_x) * tiles_x) * kBwdTile;
-    const float gx = (float)(tj + pj), gy = (float)(ti + pi);
+    // pixels past the image's edge repeat the edge's: every coordinate stays within the tile's corners
+    const int xe = min(kBwdTile - 1, u.n - 1 - tj), ye = min(kBwdTile - 1, u.n - 1 - ti);
+    const float px = (float)min(pj, xe), py0 = (float)min(pi0, ye), py1 = (float)min(pi0 + 1, ye);
+    const f32x2 np0 = f2_pack(-px, -py0), np1 = f2_pack(-px, -py1);
+    const float dy = py1 - py0;
     const T* y = static_cast<const T*>(u.in);
     const int CV = u.cfg, wd = u.wd;
-    const float inv_wd = 1.0f / (float)wd, wd_last = (float)(wd - 1);
-    const uint32_t ys_a = smem_u32(b.ys);
-    float acc = 0.0f;
+    const int wp = NC > 0 ? wd + kAdjPad : wd;   // staged values per view
+    const float inv_wp = 1.0f / (float)wp, wd_last = (float)(wd - 1);
+    const uint32_t ys_a = smem_u32(b.ys), par_a = smem_u32(b.sh->par);
+    float acc0 = 0.0f, acc1 = 0.0f;
     for (int c0 = 0; c0 < u.V; c0 += CV) {
         const int nv = min(CV, u.V - c0);
         if (tid < nv) {
-            ViewF vf = u.views[c0 + tid];
+            const ViewF vf = u.views[c0 + tid];
             int dlo;
             float r;
             bwd_view_window(vf, ti, tj, u.n, &dlo, &r);
             // every pixel's candidates [ceil(t - r), floor(t + r)] within the detector must lie in the
-            // staged window (the tile's largest t is at a corner); the loop clamps to it, so a miss is
-            // recorded, not overrun
-            const float x1 = (float)min(tj + kBwdTile - 1, u.n - 1), y1 = (float)min(ti + kBwdTile - 1, u.n - 1);
-            const float tmax = fmaxf(fmaxf(bwd_det_coord(vf, (float)tj, (float)ti), bwd_det_coord(vf, x1, (float)ti)),
-                                     fmaxf(bwd_det_coord(vf, (float)tj, y1), bwd_det_coord(vf, x1, y1)));
+            // staged window (the tile's largest t is at a corner); a miss is recorded, not overrun
+            const float x1 = (float)(tj + xe), y1 = (float)(ti + ye);
+            const float t00 = bwd_det_coord(vf, (float)tj, (float)ti), t10 = bwd_det_coord(vf, x1, (float)ti);
+            const float t01 = bwd_det_coord(vf, (float)tj, y1), t11 = bwd_det_coord(vf, x1, y1);
+            const float tmax = fmaxf(fmaxf(t00, t10), fmaxf(t01, t11)), tmin = fminf(fminf(t00, t10), fminf(t01, t11));
             if (fminf(floorf(tmax + r), (float)(u.D - 1)) > (float)(dlo + wd - 1)) record_device_error(err, RADON_ERR_DEVICE_BOUNDS);
             // every ray keeps its line in the table (a ray missing the image included)
             const int dref = min(max(dlo, 0), u.D - 1);
             const float4 A = bwd_ray_pos_rec(u.rays[(long long)(c0 + tid) * u.D + dref], true, ti, tj, u.ih2);
             // det_spacing * n = (ax, ay) / (ax^2 + ay^2): the map t = (n.P) / det_spacing + const
             const float q = 1.0f / fmaf(vf.ax, vf.ax, vf.ay * vf.ay);
-            const float2 dn = make_float2(vf.ax * q, vf.ay * q);
-            const float bx = A.z * u.ih2, by = A.w * u.ih2;
-            const float kr = fmaf(fabsf(A.z) + fabsf(A.w), u.ih2, 1e-4f);
             const float sh = (float)(dlo - dref);
-            vf.a0 -= (float)dlo;   // window-relative detector coordinate
-            b.sh->view[tid] = vf;
+            AdjView w;
+            w.nx = vf.ax * q;
+            w.ny = vf.ay * q;
+            w.bx = A.z * u.ih2;
+            w.by = A.w * u.ih2;
+            w.c = -fmaf(A.x, w.bx, A.y * w.by) - fmaf(fabsf(A.z) + fabsf(A.w), u.ih2, 1e-4f) + 0.5f;
+            w.Ax = fmaf(sh, w.nx, A.x);
+            w.Ay = fmaf(sh, w.ny, A.y);
+            w.sx = A.z;
+            w.sy = A.w;
+            w.ax = vf.ax;
+            w.ay = vf.ay;
+            w.a0 = t00 - (float)dlo;   // the tile's first pixel; r's margin covers the rounding of t00
+            if (NC > 0) {
+                // the first candidates' nearest integers stay in [0, wd - 1] (0.05 covers the rounding of
+                // the per-pixel coordinates), so the NC rays lie within the staged values
+                w.a0 = w.a0 - r + 0.5f;
+                const float lo = tmin - (float)dlo - r + 0.5f - 0.05f, hi = tmax - (float)dlo - r + 0.5f + 0.05f;
+                if (!(lo > -0.5f && hi < wd_last + 0.5f)) {   // no such window leaves the host's tables
+                    record_device_error(err, RADON_ERR_DEVICE_BOUNDS);
+                    w.ax = w.ay = w.a0 = 0.0f;
+                }
+            }
+            b.sh->par[tid] = w;
             b.sh->dlo[tid] = dlo;
             b.sh->r[tid] = r;
-            b.sh->ref[tid] = make_float4(fmaf(sh, dn.x, A.x), fmaf(sh, dn.y, A.y), A.z, A.w);
-            b.sh->bc[tid] = make_float4(bx, by, -fmaf(A.x, bx, A.y * by) - kr, 0.0f);
-            b.sh->dn[tid] = dn;
         }
         __syncthreads();
-        for (int e = tid; e < nv * wd; e += kPlanThreads) {
-            int vl = (int)((float)e * inv_wd);   // e / wd, corrected for the quotient's rounding
-            vl -= vl * wd > e;
-            vl += (vl + 1) * wd <= e;
-            const int d = b.sh->dlo[vl] + (e - vl * wd);
-            b.ys[e] = (d >= 0 && d < u.D) ? to_f32(y[(long long)(c0 + vl) * u.D + d]) : 0.0f;
+        for (int e = tid; e < nv * wp; e += kAdjThreads) {
+            int vl = (int)((float)e * inv_wp);   // e / wp, corrected for the quotient's rounding
+            vl -= vl * wp > e;
+            vl += (vl + 1) * wp <= e;
+            const int dl = e - vl * wp;
+            const int d = b.sh->dlo[vl] + dl;
+            b.ys[e] = (d >= 0 && d < u.D && dl < wd) ? to_f32(y[(long long)(c0 + vl) * u.D + d]) : 0.0f;
         }
         __syncthreads();
-        for (int vl = 0; vl < nv; ++vl) {
-            const float4 vf0 = *reinterpret_cast<const float4*>(&b.sh->view[vl]);   // ax, ay, a0 - dlo, -
-            const float r = b.sh->r[vl];
-            const float t = fmaf(vf0.x, gx, fmaf(vf0.y, gy, vf0.z));
-            // window-relative candidate range, clamped in FP32 (a non-finite coordinate still gives a
-            // loop inside the window)
-            const int la0 = __float2int_ru(fmaxf(t - r, 0.0f));
-            const int la = NC > 0 ? min(la0, wd - NC) : la0;
-            const float4 A = b.sh->ref[vl];
-            const float4 bc = b.sh->bc[vl];
-            const float2 dn = b.sh->dn[vl];
-            const float ka = ceilf(fmaf(px, bc.x, fmaf(py, bc.y, bc.z)));
-            const float fla = (float)la;
-            // sample ka of the first candidate ray, relative to the pixel
-            // (x, y) pairs advance as f32x2 (one instruction per pair); the tents stay scalar
-            f32x2 r2 = f2_pack(fmaf(ka, A.z, fmaf(fla, dn.x, A.x) - px), fmaf(ka, A.w, fmaf(fla, dn.y, A.y) - py));
-            const f32x2 st2 = f2_pack(A.z, A.w), dn2 = f2_pack(dn.x, dn.y);
-            uint32_t ya = ys_a + (uint32_t)(vl * wd + la) * 4u;
-            // one candidate ray: its KW samples' weights against the pixel, times the ray's value
-            auto candidate = [&]() {
-                f32x2 s2 = r2;
+        uint32_t va = par_a;
+        uint32_t yb = ys_a - 4u * kMagicBits;    // the magic number's bits cancel modulo 2^32
+        for (int vl = 0; vl < nv; ++vl, va += (uint32_t)sizeof(AdjView), yb += 4u * (uint32_t)wp) {
+            const float4 v0 = lds4(va), v1 = lds4(va + 16), v2 = lds4(va + 32);
+            const f32x2 A2 = f2_pack(v1.x, v1.y), st2 = f2_pack(v1.z, v1.w), dn2 = f2_pack(v2.x, v2.y);
+            const float t0 = fmaf(v0.x, px, fmaf(v0.y, py0, v0.z)), t1 = fmaf(v0.y, dy, t0);
+            const float s0 = fmaf(v2.z, px, fmaf(v2.w, py0, v0.w)), s1 = fmaf(v2.w, dy, s0);
+            const float ka0 = (s0 + kMagic) - kMagic, ka1 = (s1 + kMagic) - kMagic;
+            // one candidate ray from the sample at r2 (relative to the pixel): its KW samples' weights,
+            // (x, y) pairs advancing as f32x2 (one instruction per pair); the tents stay scalar
+            auto weight = [&](f32x2 r2) {
                 float sx, sy;
-                f2_unpack(s2, &sx, &sy);
+                f2_unpack(r2, &sx, &sy);
                 float w = __saturatef(1.0f - fabsf(sx)) * __saturatef(1.0f - fabsf(sy));
 #pragma unroll
                 for (int k = 1; k < KW; ++k) {
-                    s2 = f2_add(s2, st2);
-                    f2_unpack(s2, &sx, &sy);
+                    r2 = f2_add(r2, st2);
+                    f2_unpack(r2, &sx, &sy);
                     w = fmaf(__saturatef(1.0f - fabsf(sx)), __saturatef(1.0f - fabsf(sy)), w);
                 }
-                float yv;
-                asm volatile("ld.shared.f32 %0, [%1];" : "=f"(yv) : "r"(ya));
-                acc = fmaf(w, yv, acc);
-                r2 = f2_add(r2, dn2);
-                ya += 4u;
+                return w;
+            };
+            auto first = [&](f32x2 np, float ka, float la) {   // sample ka of ray la, relative to the pixel
+                return f2_fma(f2_pack(ka, ka), st2, f2_fma(f2_pack(la, la), dn2, f2_add(A2, np)));
             };
             if constexpr (NC > 0) {
+                const float m0 = t0 + kMagic, m1 = t1 + kMagic;
+                f32x2 ra = first(np0, ka0, m0 - kMagic), rb = first(np1, ka1, m1 - kMagic);
+                const uint32_t ya = yb + 4u * __float_as_uint(m0), yc = yb + 4u * __float_as_uint(m1);
 #pragma unroll
-                for (int c = 0; c < NC; ++c) candidate();
+                for (int c = 0; c < NC; ++c) {
+                    acc0 = fmaf(weight(ra), lds1(ya + 4u * c), acc0);
+                    acc1 = fmaf(weight(rb), lds1(yc + 4u * c), acc1);
+                    ra = f2_add(ra, dn2);
+                    rb = f2_add(rb, dn2);
+                }
             } else {
-                const int lb = __float2int_rd(fminf(t + r, wd_last));
-                for (int l = la; l <= lb; ++l) candidate();
+                // window-relative candidate ranges, clamped in FP32 (a non-finite coordinate still gives
+                // a loop inside the window)
+                const float r = b.sh->r[vl];
+                auto loop = [&](f32x2 np, float t, float ka, float& acc) {
+                    const float la = fmaxf(ceilf(t - r), 0.0f);
+                    const int lb = __float2int_rd(fminf(t + r, wd_last));
+                    f32x2 r2 = first(np, ka, la);
+                    for (int l = (int)la; l <= lb; ++l) {
+                        acc = fmaf(weight(r2), b.ys[vl * wp + l], acc);
+                        r2 = f2_add(r2, dn2);
+                    }
+                };
+                loop(np0, t0, ka0, acc0);
+                loop(np1, t1, ka1, acc1);
             }
         }
         __syncthreads();
     }
-    if ((ti + pi) < u.n && (tj + pj) < u.n) {
-        const long long idx = (long long)(ti + pi) * u.n + (tj + pj);
-        static_cast<T*>(u.out)[idx] = from_f32<T>(epilogue_value<T>(ep, u.h * acc, idx));
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        if ((ti + pi0 + x) >= u.n || (tj + pj) >= u.n) continue;
+        const long long idx = (long long)(ti + pi0 + x) * u.n + (tj + pj);
+        static_cast<T*>(u.out)[idx] = from_f32<T>(epilogue_value<T>(ep, u.h * (x ? acc1 : acc0), idx));
     }
 }
 
-// Four CTAs per SM: with both geometry kinds in one kernel the register allocation would otherwise
-// drop it to three (8.6 % slower on the uneven batch; 1.4 % faster than one generic path at four).
+// Eight CTAs of 128 threads per SM: the launch bounds keep both geometry kinds within 64 registers.
 template <typename T, int KW>
-__global__ void __launch_bounds__(kPlanThreads, 4) plan_adjoint_kernel(const Unit* __restrict__ units,
+__global__ void __launch_bounds__(kAdjThreads, 8) plan_adjoint_kernel(const Unit* __restrict__ units,
                                                                     const Work* __restrict__ work, int n_work,
                                                                     unsigned* counter, int max_wd, int cap, int* err) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -505,7 +567,7 @@ __global__ void __launch_bounds__(kPlanThreads, 4) plan_adjoint_kernel(const Uni
         const Work w = work[wi];
         const Unit& u = units[w.unit];
         if (u.fan)
-            plan_adjoint_tile<T, KW, true>(u, w.tile, b, Epilogue{1.0f, nullptr, 0.0f, nullptr}, err);
+            plan_adjoint_tile<T, KW>(u, w.tile, b, Epilogue{1.0f, nullptr, 0.0f, nullptr}, err);
         else if (u.cand3)
             plan_adjoint_tile_parallel<T, KW, 3>(u, w.tile, b, Epilogue{1.0f, nullptr, 0.0f, nullptr}, err);
         else
@@ -515,15 +577,16 @@ __global__ void __launch_bounds__(kPlanThreads, 4) plan_adjoint_kernel(const Uni
 
 // Single image (a batch-1 call): one CTA per tile, the unit passed by value.  NC < 0: fan beam.
 template <typename T, int KW, int NC>
-__global__ void __launch_bounds__(kPlanThreads) single_adjoint_kernel(const Unit u, const Epilogue ep, int* err) {
+__global__ void __launch_bounds__(kAdjThreads, 8) single_adjoint_kernel(const Unit u, const Epilogue ep, int* err) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if constexpr (NC < 0)
-        plan_adjoint_tile<T, KW, true>(u, (int)blockIdx.x, adj_buffers(smem_raw, u.wd, u.cfg), ep, err);
+        plan_adjoint_tile<T, KW>(u, (int)blockIdx.x, adj_buffers(smem_raw, u.wd, u.cfg), ep, err);
     else
         plan_adjoint_tile_parallel<T, KW, NC>(u, (int)blockIdx.x, adj_buffers(smem_raw, u.wd, u.cfg), ep, err);
 }
 
 size_t adj_smem_bytes(int max_wd, int cap) {
+    // parallel-beam units use the window constants' space past their values for the kAdjPad zeros
     return (sizeof(AdjShared) + 15) / 16 * 16 + (size_t)cap * max_wd * (16 + 4 + 4);
 }
 
@@ -717,7 +780,7 @@ radon_status single_backward_tk(const Unit& u, long long tiles, size_t smem, con
     auto kern = single_adjoint_kernel<T, KW, NC>;
     const cudaError_t ea = raise_smem_attr<single_adjoint_kernel<T, KW, NC>>(smem);
     if (ea != cudaSuccess) return cuda_fail(ea, "single-image adjoint shared memory");
-    kern<<<(unsigned)tiles, kPlanThreads, smem, s>>>(u, ep, err);
+    kern<<<(unsigned)tiles, kAdjThreads, smem, s>>>(u, ep, err);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "single-image adjoint launch");
     count_launches(1);
@@ -914,10 +977,10 @@ radon_status launch_t(const radon_plan* p, const Work* d_work, int n_work, int n
         int* err = device_error_word();
         if (err == nullptr) return fail(RADON_ERR_CUDA, "device error word unavailable");
         if (p->kw == 3)
-            plan_adjoint_kernel<T, 3><<<p->ctas, kPlanThreads, p->smem, s>>>(p->d_units, d_work, n_work, p->d_counter,
+            plan_adjoint_kernel<T, 3><<<p->ctas, kAdjThreads, p->smem, s>>>(p->d_units, d_work, n_work, p->d_counter,
                                                                             p->max_wd, p->cap, err);
         else
-            plan_adjoint_kernel<T, 6><<<p->ctas, kPlanThreads, p->smem, s>>>(p->d_units, d_work, n_work, p->d_counter,
+            plan_adjoint_kernel<T, 6><<<p->ctas, kAdjThreads, p->smem, s>>>(p->d_units, d_work, n_work, p->d_counter,
                                                                             p->max_wd, p->cap, err);
         e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "plan adjoint launch");
@@ -954,11 +1017,11 @@ radon_status occupancy_t(radon_plan* p) {
     } else if (p->kw == 3) {
         e = raise_smem_attr<plan_adjoint_kernel<T, 3>>(p->smem);
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, plan_adjoint_kernel<T, 3>, kPlanThreads, p->smem);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, plan_adjoint_kernel<T, 3>, kAdjThreads, p->smem);
     } else {
         e = raise_smem_attr<plan_adjoint_kernel<T, 6>>(p->smem);
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, plan_adjoint_kernel<T, 6>, kPlanThreads, p->smem);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, plan_adjoint_kernel<T, 6>, kAdjThreads, p->smem);
     }
     if (e != cudaSuccess) return cuda_fail(e, "plan occupancy query");
     p->ctas = std::max(1, per_sm) * sms;
