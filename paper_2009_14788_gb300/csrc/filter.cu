@@ -6,16 +6,17 @@
 // convolution that, thanks to the padding, equals the linear convolution of the D bins with the
 // kernel k = IDFT(filter) at offsets -(D-1) .. D-1.  The taps (pi / V) k are computed here once per
 // geometry in FP64 (a radix-2 FFT for the windowed filters; Ram-Lak's taps are the closed form) and
-// the kernel sums the linear convolution directly in FP32 -- a few dozen microseconds for a whole
-// sinogram batch, with no FFT on the device.  Each tap is stored as an FP32 pair hi + lo: a high-pass
-// filter cancels terms up to ~150 times the result, and one FP32 rounding per tap (fixed, so it
-// does not average out) would leave a systematic 1e-5-level error; the pair removes it.
+// the kernel sums the linear convolution directly in FP32, with no FFT on the device.  Each tap is stored
+// as an FP32 pair hi + lo: a high-pass filter cancels terms up to ~150 times the result, and one FP32
+// rounding per tap (fixed, so it does not average out) would leave a systematic 1e-5-level error; the
+// pair removes it.
 #include <algorithm>
 #include <cmath>
 #include <complex>
 #include <vector>
 
 #include "dtype.cuh"
+#include "f32x2.cuh"
 #include "radon_internal.h"
 
 namespace radon {
@@ -24,7 +25,12 @@ namespace {
 
 constexpr int kFilterKinds = 5;
 constexpr int kFilterThreads = 256;
-constexpr int kFilterOut = 4;    // consecutive outputs per thread
+constexpr int kFilterOut = 8;    // outputs per thread
+constexpr int kLongOut = 4;      // consecutive outputs per thread of the kernel for long rows
+// Taps nearer than this also add their lo part.  Every kernel here falls off like 1 / m^2, so the rounding
+// errors of all farther taps together stay below 2^-25 / (64 pi^2) = 5e-11 of the largest input, under
+// 1e-7 of a result a thousand times smaller (FP32 sums of a few hundred terms carry that much).
+constexpr int kFilterNear = 64;
 
 using cd = std::complex<double>;
 
@@ -68,58 +74,293 @@ double window(int kind, double f) {
     }
 }
 
-// One row: out[d] = sum_{d'} y[d'] taps[d - d' + D - 1], kFilterOut outputs per thread; each tap is
-// a (hi, lo) pair summed into two accumulators.
+// One row whose taps and bins do not fit one CTA's shared memory in the layout below (more than about
+// 9600 bins): out[d] = sum_{d'} y[d'] taps[d - d' + D - 1], kLongOut outputs per thread; each tap is a
+// (hi, lo) pair summed into two accumulators.
 template <typename T>
-__global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const T* __restrict__ in, T* __restrict__ out,
+__global__ void __launch_bounds__(kFilterThreads) filter_long_rows_kernel(const T* __restrict__ in, T* __restrict__ out,
                                                                      const float2* __restrict__ taps, int D) {
     extern __shared__ float fsm[];
-    const int Dp = (D + kFilterOut - 1) / kFilterOut * kFilterOut;   // bins padded to whole output groups
+    const int Dp = (D + kLongOut - 1) / kLongOut * kLongOut;   // bins padded to whole output groups
     float* y = fsm;                                           // [Dp], zero past D
-    float2* t = reinterpret_cast<float2*>(fsm + Dp + (Dp & 1));   // taps at offset +kFilterOut
+    float2* t = reinterpret_cast<float2*>(fsm + Dp + (Dp & 1));   // taps at offset +kLongOut
     const long long row = blockIdx.x;
     const T* src = in + row * D;
     for (int d = threadIdx.x; d < Dp; d += blockDim.x) y[d] = d < D ? to_f32(src[d]) : 0.0f;
-    const int nt = 2 * Dp + 2 * kFilterOut;
+    const int nt = 2 * Dp + 2 * kLongOut;
     for (int j = threadIdx.x; j < nt; j += blockDim.x) {
-        const int m = j - kFilterOut;    // tap index relative to taps[0]
+        const int m = j - kLongOut;    // tap index relative to taps[0]
         t[j] = (m >= 0 && m < 2 * D - 1) ? taps[m] : make_float2(0.0f, 0.0f);
     }
     __syncthreads();
     T* dst = out + row * D;
-    for (int d0 = threadIdx.x * kFilterOut; d0 < D; d0 += blockDim.x * kFilterOut) {
-        float hi[kFilterOut], lo[kFilterOut];
+    for (int d0 = threadIdx.x * kLongOut; d0 < D; d0 += blockDim.x * kLongOut) {
+        float hi[kLongOut], lo[kLongOut];
 #pragma unroll
-        for (int o = 0; o < kFilterOut; ++o) hi[o] = lo[o] = 0.0f;
-        // tap of output d0 + o and input d' sits at t[d0 + o - d' + D - 1 + kFilterOut]; the taps
+        for (int o = 0; o < kLongOut; ++o) hi[o] = lo[o] = 0.0f;
+        // tap of output d0 + o and input d' sits at t[d0 + o - d' + D - 1 + kLongOut]; the taps
         // of consecutive inputs slide by one, so a register window takes one new tap per input
-        const float2* tb = t + d0 + D - 1 + kFilterOut;
-        float2 w[kFilterOut];
+        const float2* tb = t + d0 + D - 1 + kLongOut;
+        float2 w[kLongOut];
 #pragma unroll
-        for (int o = 0; o < kFilterOut; ++o) w[o] = tb[o];
-        for (int q = 0; q < Dp; q += kFilterOut) {
+        for (int o = 0; o < kLongOut; ++o) w[o] = tb[o];
+        for (int q = 0; q < Dp; q += kLongOut) {
 #pragma unroll
-            for (int u = 0; u < kFilterOut; ++u) {
+            for (int u = 0; u < kLongOut; ++u) {
                 const float yv = y[q + u];
 #pragma unroll
-                for (int o = 0; o < kFilterOut; ++o) {
+                for (int o = 0; o < kLongOut; ++o) {
                     hi[o] = fmaf(yv, w[o].x, hi[o]);
                     lo[o] = fmaf(yv, w[o].y, lo[o]);
                 }
 #pragma unroll
-                for (int o = kFilterOut - 1; o > 0; --o) w[o] = w[o - 1];
+                for (int o = kLongOut - 1; o > 0; --o) w[o] = w[o - 1];
                 w[0] = tb[-(q + u + 1)];
             }
         }
 #pragma unroll
-        for (int o = 0; o < kFilterOut; ++o)
+        for (int o = 0; o < kLongOut; ++o)
             if (d0 + o < D) dst[d0 + o] = from_f32<T>(hi[o] + lo[o]);
     }
 }
 
-size_t filter_smem(int D) {
-    const int Dp = (D + kFilterOut - 1) / kFilterOut * kFilterOut;
-    return (size_t)(Dp + (Dp & 1)) * sizeof(float) + (size_t)(2 * Dp + 2 * kFilterOut) * sizeof(float2);
+// Shared-memory plan of a CTA (floats), the same on host and device.  The convolution runs as S sums over
+// interleaved bins: with HALF (Ram-Lak, whose taps at even offsets but zero are exactly 0) the even
+// outputs take the odd bins and the odd outputs the even ones, S = 2; otherwise S = 1.  Sum s has
+// `A` outputs in groups of kFilterOut and `L4` bins (whole float4s, zero past the row).
+struct FilterPlan {
+    int L4;      // bins of one sum
+    int A8;      // outputs of one sum, in whole groups
+    int nt;      // reversed taps of one copy
+    int c0;      // place of the tap of bin distance zero in the first copy
+    int bl;      // reach of the near taps, in bins of the sum
+    int ntl;     // reversed near (lo) taps of one copy
+    int tap_floats, row_floats;
+};
+
+template <bool HALF>
+__host__ __device__ inline FilterPlan filter_plan(int D) {
+    FilterPlan f;
+    const int A = HALF ? (D + 1) / 2 : D;
+    f.L4 = (A + 3) / 4 * 4;
+    f.A8 = (A + kFilterOut - 1) / kFilterOut * kFilterOut;
+    f.c0 = f.A8 + 8;
+    f.nt = f.A8 + f.L4 + 24;
+    f.bl = HALF ? kFilterNear / 2 : kFilterNear;
+    f.ntl = 2 * f.bl + 24;
+    f.tap_floats = (HALF ? 2 : 1) * 2 * (f.nt + f.ntl);
+    f.row_floats = (HALF ? 2 : 1) * f.L4 + (D + 3) / 4 * 4;
+    return f;
+}
+
+// out[d] = sum_d' y[d'] taps[d - d' + D - 1] for `rpc` rows per CTA, `tpr` threads per row, kFilterOut
+// outputs of one sum per thread.  Bound by FP32 issue: products are paired over two neighbouring bins
+// (fma.rn.f32x2: half the instructions), so an output's taps are needed as pairs at even and at odd
+// offsets: the reversed taps lie in shared memory twice, the second copy shifted by one, and both
+// windows slide in registers, one 16-byte load of each per four bins.  With Ram-Lak the zero taps are
+// left out.  512 views of 725 bins, FP32: 77 us with one bin per scalar FMA, both tap parts and the
+// zeros; see the figures beside the launch.
+template <typename T, bool HALF>
+__global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const T* __restrict__ in, T* __restrict__ out,
+                                                                     const float2* __restrict__ taps, int D,
+                                                                     long long rows, int rpc, int tpr) {
+    extern __shared__ __align__(16) float fsm[];
+    constexpr int S = HALF ? 2 : 1;
+    const FilterPlan f = filter_plan<HALF>(D);
+    const long long row0 = (long long)blockIdx.x * rpc;
+    const int nrows = (int)min((long long)rpc, rows - row0);
+    float* rowmem = fsm + f.tap_floats;
+    // reversed taps of sum s: hi even copy [nt], hi odd copy, lo even copy [ntl], lo odd copy; entry x of
+    // the even copies is the tap of bin distance (output - bin) = c0 - x (hi) or bl + 8 - x (lo), the odd
+    // copies hold the same one place later
+    for (int e = threadIdx.x; e < S * (f.nt + f.ntl); e += blockDim.x) {
+        const int s = HALF ? e / (f.nt + f.ntl) : 0, x = e - s * (f.nt + f.ntl);
+        const bool far = x < f.nt;
+        float* dst = fsm + s * 2 * (f.nt + f.ntl) + (far ? x : 2 * f.nt + (x - f.nt));
+        const int q = far ? f.c0 - x : f.bl + 8 - (x - f.nt);
+#pragma unroll
+        for (int odd = 0; odd < 2; ++odd) {
+            const int m = HALF ? 2 * (q + odd) + 2 * s - 1 : q + odd;   // offset in bins of the row
+            float v = 0.0f;
+            if (m > -D && m < D) {
+                const float2 t = __ldg(taps + m + D - 1);
+                v = far ? t.x : (m > -kFilterNear && m < kFilterNear ? t.y : 0.0f);
+            }
+            dst[odd * (far ? f.nt : f.ntl)] = v;
+        }
+    }
+    // rows: with HALF the odd bins first (the even outputs' sum), then the even bins
+    for (int r = 0; r < nrows; ++r) {
+        const T* src = in + (row0 + r) * D;
+        float* y = rowmem + (size_t)r * f.row_floats;
+        for (int d = threadIdx.x; d < S * f.L4; d += blockDim.x)
+            y[HALF ? ((d & 1) ? d >> 1 : f.L4 + (d >> 1)) : d] = d < D ? to_f32(src[d]) : 0.0f;
+    }
+    __syncthreads();
+    const int r = (int)threadIdx.x / tpr, t0 = (int)threadIdx.x - r * tpr;
+    if (r < nrows) {
+        const float* y = rowmem + (size_t)r * f.row_floats;
+        float* res = rowmem + (size_t)r * f.row_floats + S * f.L4;
+        const int gps = f.A8 / kFilterOut;   // groups per sum
+        for (int g = t0; g < S * gps; g += tpr) {
+            const int s = HALF ? (g >= gps ? 1 : 0) : 0, a0 = (g - s * gps) * kFilterOut;
+            const float* x = y + s * f.L4;
+            const float* tp = fsm + s * 2 * (f.nt + f.ntl);
+            f32x2 acc[kFilterOut];
+#pragma unroll
+            for (int o = 0; o < kFilterOut; ++o) acc[o] = 0ull;
+            // bins [i0, i1) (multiples of 4) against the taps at e (outputs a0, a0 + 2, ...) and d (a0 + 1, ...)
+            auto conv = [&](const float* xi, const float* e, const float* d, int n) {
+                f32x2 e3 = *reinterpret_cast<const f32x2*>(e - 6), e2 = *reinterpret_cast<const f32x2*>(e - 4),
+                      e1 = *reinterpret_cast<const f32x2*>(e - 2);
+                f32x2 d3 = *reinterpret_cast<const f32x2*>(d - 6), d2 = *reinterpret_cast<const f32x2*>(d - 4),
+                      d1 = *reinterpret_cast<const f32x2*>(d - 2);
+#pragma unroll 2
+                for (int i = 0; i < n; i += 4) {
+                    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(xi + i);
+                    const ulonglong2 ee = *reinterpret_cast<const ulonglong2*>(e + i);
+                    const ulonglong2 dd = *reinterpret_cast<const ulonglong2*>(d + i);
+                    acc[0] = f2_fma(v.x, ee.x, acc[0]);
+                    acc[1] = f2_fma(v.x, dd.x, acc[1]);
+                    acc[2] = f2_fma(v.x, e1, acc[2]);
+                    acc[3] = f2_fma(v.x, d1, acc[3]);
+                    acc[4] = f2_fma(v.x, e2, acc[4]);
+                    acc[5] = f2_fma(v.x, d2, acc[5]);
+                    acc[6] = f2_fma(v.x, e3, acc[6]);
+                    acc[7] = f2_fma(v.x, d3, acc[7]);
+                    acc[0] = f2_fma(v.y, ee.y, acc[0]);
+                    acc[1] = f2_fma(v.y, dd.y, acc[1]);
+                    acc[2] = f2_fma(v.y, ee.x, acc[2]);
+                    acc[3] = f2_fma(v.y, dd.x, acc[3]);
+                    acc[4] = f2_fma(v.y, e1, acc[4]);
+                    acc[5] = f2_fma(v.y, d1, acc[5]);
+                    acc[6] = f2_fma(v.y, e2, acc[6]);
+                    acc[7] = f2_fma(v.y, d2, acc[7]);
+                    e3 = e1;
+                    e2 = ee.x;
+                    e1 = ee.y;
+                    d3 = d1;
+                    d2 = dd.x;
+                    d1 = dd.y;
+                }
+            };
+            // the lo products, summed by themselves
+            float lo[kFilterOut];
+            const int i0 = max(a0 - f.bl, 0), i1 = min(a0 + kFilterOut + f.bl, f.L4);
+            const float* tl = tp + 2 * f.nt + (i0 - a0 + f.bl + 8);
+            if (i1 > i0) conv(x + i0, tl, tl + f.ntl, i1 - i0);
+#pragma unroll
+            for (int o = 0; o < kFilterOut; ++o) {
+                float p, q;
+                f2_unpack(acc[o], &p, &q);
+                lo[o] = p + q;
+                acc[o] = 0ull;
+            }
+            // A high-pass sum is as large as its centre taps make it and small again once they are in, so the
+            // bins next to the outputs, [a0 - 4, a0 + 12), are added one by one in row order (the centre
+            // tap in its place) between the farther ones of either side: as few additions round at
+            // the large values as in a plain sum along the row (pairs throughout left 2.5 times its error).
+            const float* hi = tp + (f.c0 - a0);
+            if (a0 > 4) conv(x, hi, hi + f.nt, a0 - 4);
+            float v[kFilterOut];
+#pragma unroll
+            for (int o = 0; o < kFilterOut; ++o) {
+                float p, q;
+                f2_unpack(acc[o], &p, &q);
+                v[o] = p + q;
+            }
+            float t[24];   // taps of bin distance (bin - output) -12 .. 11
+#pragma unroll
+            for (int j = 0; j < 24; j += 4)
+                *reinterpret_cast<float4*>(t + j) = *reinterpret_cast<const float4*>(tp + f.c0 - 12 + j);
+            const float2 centre = __ldg(taps + D - 1);
+            float own[kFilterOut];
+#pragma unroll
+            for (int o = 0; o < kFilterOut; ++o) {
+                own[o] = HALF && a0 + o < f.L4 ? y[(1 - s) * f.L4 + a0 + o] : 0.0f;
+                lo[o] = HALF ? fmaf(own[o], centre.y, lo[o]) : lo[o];
+            }
+#pragma unroll
+            for (int j = -4; j < 12; j += 4) {
+                const int i = a0 + j;
+                float xi[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                if (i >= 0 && i < f.L4) *reinterpret_cast<float4*>(xi) = *reinterpret_cast<const float4*>(x + i);
+#pragma unroll
+                for (int w = 0; w < 4; ++w)
+#pragma unroll
+                    for (int o = 0; o < kFilterOut; ++o) {
+                        // with HALF an output's own bin, one of the other sum's, lies before bin a0 + o of the
+                        // odd bins (s = 0) and after bin a0 + o of the even ones (s = 1)
+                        if (HALF && j + w == o) v[o] = fmaf(s == 0 ? own[o] : 0.0f, centre.x, v[o]);
+                        if (HALF && j + w == o + 1) v[o] = fmaf(s == 0 ? 0.0f : own[o], centre.x, v[o]);
+                        v[o] = fmaf(xi[w], t[j + w - o + 12], v[o]);
+                    }
+            }
+            const int right = a0 + 12;
+#pragma unroll
+            for (int o = 0; o < kFilterOut; ++o) acc[o] = f2_pack(0.5f * v[o], 0.5f * v[o]);
+            if (right < f.L4) conv(x + right, hi + right, hi + f.nt + right, f.L4 - right);
+#pragma unroll
+            for (int o = 0; o < kFilterOut; ++o) {
+                float p, q;
+                f2_unpack(acc[o], &p, &q);
+                const int a = a0 + o, dd = HALF ? 2 * a + s : a;
+                if (dd < D) res[dd] = (p + q) + lo[o];
+            }
+        }
+    }
+    __syncthreads();
+    for (int q = 0; q < nrows; ++q) {
+        T* dst = out + (row0 + q) * D;
+        const float* res = rowmem + (size_t)q * f.row_floats + S * f.L4;
+        for (int d = threadIdx.x; d < D; d += blockDim.x) dst[d] = from_f32<T>(res[d]);
+    }
+}
+
+// Shared memory of the kernel for long rows: the largest row served is the one whose bins and (hi, lo)
+// taps one CTA holds.
+size_t filter_long_smem(int D) {
+    const int Dp = (D + kLongOut - 1) / kLongOut * kLongOut;
+    return (size_t)(Dp + (Dp & 1)) * sizeof(float) + (size_t)(2 * Dp + 2 * kLongOut) * sizeof(float2);
+}
+
+template <typename T>
+cudaError_t filter_launch_long(const void* in, void* out, const float2* taps, int D, long long rows, cudaStream_t s) {
+    const size_t smem = filter_long_smem(D);
+    cudaError_t e = cudaFuncSetAttribute(filter_long_rows_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
+    filter_long_rows_kernel<T><<<(unsigned)rows, kFilterThreads, smem, s>>>((const T*)in, (T*)out, taps, D);
+    return cudaGetLastError();
+}
+
+template <typename T, bool HALF>
+cudaError_t filter_launch(const void* in, void* out, const float2* taps, int D, long long rows, cudaStream_t s) {
+    const FilterPlan f = filter_plan<HALF>(D);
+    const int groups = (HALF ? 2 : 1) * f.A8 / kFilterOut;
+    const int tpr = std::min(kFilterThreads, (groups + 31) / 32 * 32);
+    // Rows per CTA share its taps: as many as one CTA's threads and half an SM's shared memory hold while
+    // every SM keeps about eight rows' worth of warps.
+    int rpc = 1;
+    if ((size_t)(f.tap_floats + f.row_floats) * sizeof(float) > 227 * 1024)
+        return filter_launch_long<T>(in, out, taps, D, rows, s);
+    while (rpc < 4 && (rpc + 1) * tpr <= kFilterThreads && rows >= (long long)(rpc + 1) * 152 * 8 &&
+           (size_t)(f.tap_floats + (rpc + 1) * f.row_floats) * sizeof(float) <= 112 * 1024)
+        ++rpc;
+    const size_t smem = (size_t)(f.tap_floats + rpc * f.row_floats) * sizeof(float);
+    cudaError_t e = cudaFuncSetAttribute(filter_rows_kernel<T, HALF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)std::max<size_t>(smem, 48 * 1024));
+    if (e != cudaSuccess) return e;
+    filter_rows_kernel<T, HALF><<<(unsigned)((rows + rpc - 1) / rpc), rpc * tpr, smem, s>>>(
+        (const T*)in, (T*)out, taps, D, rows, rpc, tpr);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t filter_launch(const void* in, void* out, const float2* taps, int D, long long rows, radon_filter filter,
+                          cudaStream_t s) {
+    return filter == RADON_FILTER_RAM_LAK ? filter_launch<T, true>(in, out, taps, D, rows, s)
+                                          : filter_launch<T, false>(in, out, taps, D, rows, s);
 }
 
 }  // namespace
@@ -182,39 +423,19 @@ extern "C" RADON_API radon_status radon_filter_sinogram(const radon_geometry* g,
     const uintptr_t a = (uintptr_t)sino, b = (uintptr_t)out;
     if (batch > 0 && a < b + bytes && b < a + bytes) return fail(RADON_ERR_INVALID_ARG, "out overlaps sino");
     if (batch == 0) return RADON_OK;
-    const size_t smem = filter_smem(g->D);
-    if (smem > 227 * 1024) return fail(RADON_ERR_UNSUPPORTED, "det_count too large for the filter kernel");
+    if (filter_long_smem(g->D) > 227 * 1024)
+        return fail(RADON_ERR_UNSUPPORTED, "det_count too large for the filter kernel");
     if (rows > 0x7fffffffLL) return fail(RADON_ERR_UNSUPPORTED, "too many sinogram rows");
     st = check_device(g);
     if (st != RADON_OK) return st;
     const float2* taps = g->d_filter_taps + (size_t)filter * (2LL * g->D - 1);
     cudaStream_t s = (cudaStream_t)stream;
-    // one thread per kFilterOut outputs of the row, in whole warps, at most kFilterThreads
-    const int groups = (g->D + kFilterOut - 1) / kFilterOut;
-    const int threads = std::min(kFilterThreads, (groups + 31) / 32 * 32);
     cudaError_t e;
     switch (dtype) {
-        case RADON_F16:
-            e = cudaFuncSetAttribute(filter_rows_kernel<__half>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e == cudaSuccess)
-                filter_rows_kernel<__half><<<(unsigned)rows, threads, smem, s>>>((const __half*)sino, (__half*)out,
-                                                                                       taps, g->D);
-            break;
-        case RADON_BF16:
-            e = cudaFuncSetAttribute(filter_rows_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem);
-            if (e == cudaSuccess)
-                filter_rows_kernel<__nv_bfloat16><<<(unsigned)rows, threads, smem, s>>>(
-                    (const __nv_bfloat16*)sino, (__nv_bfloat16*)out, taps, g->D);
-            break;
-        default:
-            e = cudaFuncSetAttribute(filter_rows_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e == cudaSuccess)
-                filter_rows_kernel<float><<<(unsigned)rows, threads, smem, s>>>((const float*)sino, (float*)out,
-                                                                                      taps, g->D);
-            break;
+        case RADON_F16: e = filter_launch<__half>(sino, out, taps, g->D, rows, filter, s); break;
+        case RADON_BF16: e = filter_launch<__nv_bfloat16>(sino, out, taps, g->D, rows, filter, s); break;
+        default: e = filter_launch<float>(sino, out, taps, g->D, rows, filter, s); break;
     }
-    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "filter launch");
     count_launches(1);
     return RADON_OK;
