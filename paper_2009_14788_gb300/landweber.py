@@ -10,7 +10,9 @@ Reverse mode with per-iteration checkpointing: the forward pass keeps only the i
 backward pass recomputes each residual and runs, for k = K-1 .. 0 (g_K = dL/dx_K),
     t = A g_{k+1};   dL/dalpha -= <t, r_k>   (= <g_{k+1}, A^T r_k>, the adjoint identity);
     dL/dy += alpha t;   g_k = g_{k+1} - alpha A^T t,
-and dL/dx_0 = g_0.  Each backward step is three projections, one inner product and one scaled add.
+and dL/dx_0 = g_0.  Each backward step is three projections, one inner product and one scaled add; what
+only serves a gradient that nobody asked for is left out (r_k and the inner product without dL/dalpha,
+the sum without dL/dy, the last adjoint without dL/dx_0).
 """
 
 from __future__ import annotations
@@ -79,27 +81,30 @@ class LandweberFunction(torch.autograd.Function):
         bufs = _Buffers(geom, y.dtype, batch, y.device)
         g = torch.empty_like(xs[0] if xs else grad)
         axpby(grad.contiguous(), g, 1.0, beta=0.0)            # g_K (a private copy, updated in place)
+        need_y, need_a, need_x = ctx.needs_input_grad[:3]
         dalpha = torch.zeros(1, dtype=torch.float32, device=y.device) if K == 0 else \
             torch.empty(1, dtype=torch.float32, device=y.device)
-        dy32 = torch.empty(y.shape, dtype=torch.float32, device=y.device)
-        if K == 0:
+        dy32 = torch.empty(y.shape, dtype=torch.float32, device=y.device) if need_y else None
+        if K == 0 and need_y:
             axpby(y, dy32, 0.0, beta=0.0)
-        r = torch.empty_like(y)
+        r = torch.empty_like(y) if need_a else None
         t = torch.empty_like(y)
         for k in range(K - 1, -1, -1):
             first = k == K - 1
-            bufs.fwd(geom, xs[k], add=y, add_scale=-1.0, out=r, config=config)       # r_k (recomputed)
             bufs.fwd(geom, g, out=t, config=config)                                 # t = A g_{k+1}
-            dot(t, r, result=dalpha, scale=-1.0, accumulate=not first, workspace=bufs.dws)
-            axpby(t, dy32, 1.0, alpha_dev=a, beta=0.0 if first else 1.0)            # dy += alpha t
-            bufs.adj(geom, t, op_scale=-1.0, op_scale_dev=a, add=g, add_scale=1.0, out=g,
-                     config=config)                                                  # g_k in place
+            if need_a:
+                bufs.fwd(geom, xs[k], add=y, add_scale=-1.0, out=r, config=config)   # r_k (recomputed)
+                dot(t, r, result=dalpha, scale=-1.0, accumulate=not first, workspace=bufs.dws)
+            if need_y:
+                axpby(t, dy32, 1.0, alpha_dev=a, beta=0.0 if first else 1.0)        # dy += alpha t
+            if k > 0 or need_x:
+                bufs.adj(geom, t, op_scale=-1.0, op_scale_dev=a, add=g, add_scale=1.0, out=g,
+                         config=config)                                              # g_k in place
         dy = None
-        if ctx.needs_input_grad[0]:
+        if need_y:
             dy = torch.empty_like(y)
             axpby(dy32, dy, 1.0, beta=0.0)
-        return dy, dalpha.reshape(a.shape) if ctx.needs_input_grad[1] else None, \
-            g if ctx.needs_input_grad[2] else None, None, None, None
+        return dy, dalpha.reshape(a.shape) if need_a else None, g if need_x else None, None, None, None
 
 
 class Landweber:
