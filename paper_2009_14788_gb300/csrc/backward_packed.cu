@@ -56,8 +56,9 @@ int backward_packed_images_per_cta(const radon_geometry* g, int batch, radon_dty
     // than 32-image groups computing them (parallel 32 x 512^2, 512 views, FP16 adjoint: 1.84 vs 1.94
     // ms; FP32 rows measured no faster: a step of 4.32 vs 4.27 ms)
     if (g->d_tab_w != nullptr && dt != RADON_F32) return 16;
-    // A 32-image CTA costs ~1.56x a 16-image one (each weight serves twice the images; two CTAs per
-    // SM): take it when its groups cost less and its staging fits one CTA's shared memory.
+    // A 32-image CTA costs about 1.56x a 16-image one (1.38x on parallel 512^2 with 512 views, 1.6x on
+    // 360-view fans with 1024 detectors): take it when its groups cost less and its staging fits one CTA's
+    // shared memory.
     const long long g32 = (batch + 31) / 32, g16 = (batch + 15) / 16;
     if (25 * g32 < 16 * g16 && smem_32(g, dt) <= 227 * 1024) return 32;
     return 16;

@@ -8,13 +8,12 @@
 //   * the producer warp computes each view's detector window for the tile (and checks that it holds
 //     every pixel's candidate rays), then issues per view one TMA copy of the window's rows
 //     [det][BG] and one of the window's rows of the ray table, up to the ring's depth ahead;
-//   * the 256 consumer threads (one pixel each), once a chunk has landed, convert 16-bit windows to
+//   * the 128 consumer threads, once a chunk has landed, convert 16-bit windows to
 //     FP32 rows of pitch (BG + 4) words in a double buffer (FP32 windows land in that layout
 //     directly), re-base each landed ray on the tile in place -- reference sample, step and the
 //     window constant C of its candidate samples -- meet at a named barrier and gather: each thread
-//     owns two vertically neighbouring pixels (one for 32-image groups); for every candidate ray of
-//     either pixel, each pixel's KW sample weights once for all BG images, then one FP32 FMA per
-//     image and pixel from one row of loads.
+//     owns two vertically neighbouring pixels; for every candidate ray of either pixel, each pixel's KW
+//     sample weights once for all BG images, then one FP32 FMA per image and pixel from one row of loads.
 // Shared-memory addresses stay 32-bit (explicit ld/st.shared), and no index needs a division.
 // The row pitch of (BG + 4) words is an odd number of 16-byte units, so the 16-byte loads of eight
 // lanes that read eight consecutive detectors fall in eight different bank groups.
@@ -34,15 +33,17 @@ namespace radon {
 
 constexpr int kBwdPViews = 4;            // views per chunk
 constexpr int kBwdPMaxStages = 4;        // ring depth limit (mbarrier slots in the header)
-// Pixels per consumer thread: a vertical pair of neighbours shares its candidate rays, so every ray
-// record and window row loaded from shared memory serves both pixels' accumulators (16-image groups);
-// 32-image groups keep one pixel per thread (their accumulators already fill the registers).
+// A consumer thread owns a vertical pair of pixels, which share their candidate rays: every ray record
+// and window row loaded from shared memory serves both pixels' accumulators.  For 32-image groups the pair
+// fills 127 registers at three CTAs per SM (two pixels x 32 sums); one pixel per thread, four CTAs' worth
+// of warps, read every row twice as often: parallel 32 x 512^2, 512 views, FP16 1.92 -> 1.70 ms, and
+// 1.54 ms with the records' second half cut to the one word that cannot be recomputed.
 template <int BG>
 struct BwdPShape {
-    static constexpr int PX = BG <= 16 ? 2 : 1;
+    static constexpr int PX = 2;
     static constexpr int kConsumers = kBwdThreads / PX;
     static constexpr int kThreads = kConsumers + 32;
-    static constexpr int kCtasPerSm = PX == 2 ? 4 : 2;   // resident CTAs the launch bounds ask for
+    static constexpr int kCtasPerSm = BG <= 16 ? 4 : 3;   // resident CTAs the launch bounds ask for
 };
 constexpr size_t kBwdPHeader = 1024;     // barriers, flags, windows and view maps of the ring
 
@@ -100,7 +101,7 @@ struct BwdPArgs {
 };
 
 // Weight table of the exact adjoint (the TAB mode of the packed kernel): per 16 x 16 tile, view and
-// consumer thread (a vertical pixel pair, the PX = 2 layout) the detector index la of the first ray
+// consumer thread (a vertical pixel pair, the packed adjoint's layout) the detector index la of the first ray
 // that weighs on either pixel and both pixels' weights on rays la .. la + 4 (zero past the pair's
 // candidates), or la = kBwdTabOverflow where the pair's weighted rays span more than five detectors
 // (rays much denser than a pixel) -- such pairs compute their weights as without a table.  (On the
@@ -112,7 +113,7 @@ constexpr int kBwdTabRays = 5;
 constexpr int kBwdTabOverflow = (int)0x80000000;
 constexpr int kBwdTabPairs = kBwdThreads / 2;   // consumer threads of a 16-image CTA
 
-// Pixel pair of consumer thread `tid` in a 16 x 16 tile (PX = 2): rows pi0, pi0 + 1 of column pj.
+// Pixel pair of consumer thread `tid` in a 16 x 16 tile: rows pi0, pi0 + 1 of column pj.
 // Each warp takes an 8 x 8 block, each group of eight lanes a 4 x 4 block (2 x 4 pairs).
 __host__ __device__ inline void bwdp_pair_of(int tid, int* pi0, int* pj) {
     const int warp = tid >> 5, lane = tid & 31;
@@ -184,7 +185,7 @@ __device__ __forceinline__ void bwdp_widen8<__nv_bfloat16>(const uint4 u, float4
                          __uint_as_float(u.w & 0xffff0000u));
 }
 
-// TAB (exact adjoint, PX = 2 only): a pair's weights come from the geometry's weight table instead of
+// TAB (exact adjoint, groups of 8 and 16 images): a pair's weights come from the geometry's weight table instead of
 // being evaluated from re-based ray records; ray rows are copied and re-based only for chunks with a
 // view in which some pair of the tile overflows the table (the table's per-view flags).  The producer
 // prefetches the table's rows for the chunk that will next reuse its ring slot into L2.
@@ -192,7 +193,7 @@ template <typename T, int BG, int KW, bool TAB = false>
 __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasPerSm)
     backward_packed_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap rmap,
                            const BwdPArgs a) {
-    static_assert(!TAB || (KW > 0 && BwdPShape<BG>::PX == 2), "the weight table serves the exact adjoint's pairs");
+    static_assert(!TAB || (KW > 0 && BG <= 16), "the weight table serves the exact adjoint's smaller groups");
     constexpr bool kRays = KW > 0;   // ray rows copied and re-based per chunk
     using L = BwdPLayout<T, BG>;
     constexpr int NQ = BG / 4;
@@ -301,15 +302,12 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
     }
 
     // ---------------------------------------------------------------------- consumer warps
-    // each warp takes an (4 PX) x 8 block of the tile, lanes on a 4 x 8 grid of pixels (PX = 1) or
-    // vertical pixel pairs (PX = 2): a block's detector footprints overlap more than those of a strip,
-    // so the gather's shared loads touch fewer distinct addresses.  A 16-byte shared load is served
-    // eight lanes at a time, so each group of eight lanes covers a compact block -- 4 x 2 pixels, or
-    // 2 x 4 pairs (4 x 4 pixels) -- whose detector span stays within the eight bank groups
-    const int warp = tid >> 5, lane = tid & 31;
-    const int grp = lane >> 3, e8 = lane & 7;
-    int pi0 = (warp >> 1) * 4 + (e8 >> 1), pj = (warp & 1) * 8 + grp * 2 + (e8 & 1);
-    if constexpr (PX == 2) bwdp_pair_of(tid, &pi0, &pj);
+    // each warp takes an 8 x 8 block of the tile, lanes on a 4 x 8 grid of vertical pixel pairs: a block's
+    // detector footprints overlap more than those of a strip, so the gather's shared loads touch fewer
+    // distinct addresses.  A 16-byte shared load is served eight lanes at a time, so each group of eight
+    // lanes covers a compact block of 2 x 4 pairs, whose detector span stays within the eight bank groups
+    int pi0, pj;
+    bwdp_pair_of(tid, &pi0, &pj);
     const float px = (float)pj, py0 = (float)pi0;
     const float gx = (float)(tj + pj), gy0 = (float)(ti + pi0);
     float acc[PX][BG];
@@ -387,7 +385,7 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
                     float4 A, Bc;
                     bwdp_rebase(ray, d >= 0 && d < a.D, ti, tj, a.ih2, &A, &Bc);
                     sts4(rec, A);
-                    sts4(rec + 16, Bc);
+                    sts1(rec + 16, Bc.z);
                 }
             }
         }
@@ -497,16 +495,16 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
                                 const f32x2 y01 = f2_pack(y4.x, y4.y), y23 = f2_pack(y4.z, y4.w);
                                 f32x2 a0 = f2_pack(acc[0][4 * q + 0], acc[0][4 * q + 1]);
                                 f32x2 a1 = f2_pack(acc[0][4 * q + 2], acc[0][4 * q + 3]);
-                                f32x2 b0 = f2_pack(acc[PX - 1][4 * q + 0], acc[PX - 1][4 * q + 1]);
-                                f32x2 b1 = f2_pack(acc[PX - 1][4 * q + 2], acc[PX - 1][4 * q + 3]);
+                                f32x2 b0 = f2_pack(acc[1][4 * q + 0], acc[1][4 * q + 1]);
+                                f32x2 b1 = f2_pack(acc[1][4 * q + 2], acc[1][4 * q + 3]);
                                 a0 = f2_fma(wwa, y01, a0);
                                 a1 = f2_fma(wwa, y23, a1);
                                 b0 = f2_fma(wwb, y01, b0);
                                 b1 = f2_fma(wwb, y23, b1);
                                 f2_unpack(a0, &acc[0][4 * q + 0], &acc[0][4 * q + 1]);
                                 f2_unpack(a1, &acc[0][4 * q + 2], &acc[0][4 * q + 3]);
-                                f2_unpack(b0, &acc[PX - 1][4 * q + 0], &acc[PX - 1][4 * q + 1]);
-                                f2_unpack(b1, &acc[PX - 1][4 * q + 2], &acc[PX - 1][4 * q + 3]);
+                                f2_unpack(b0, &acc[1][4 * q + 0], &acc[1][4 * q + 1]);
+                                f2_unpack(b1, &acc[1][4 * q + 2], &acc[1][4 * q + 3]);
                             }
                         }
                     }
@@ -520,28 +518,28 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
                     // that it holds them all); the bounds are clamped in FP32, so a non-finite coordinate
                     // still gives a loop inside the window
                     float tlo = __fdividef(num0, den0), thi = tlo;
-                    if constexpr (PX == 2) {
-                        const float t1 = __fdividef(num0 + v01.y, den0 + v23.x);
-                        tlo = fminf(tlo, t1);
-                        thi = fmaxf(thi, t1);
-                    }
+                    const float t1 = __fdividef(num0 + v01.y, den0 + v23.x);
+                    tlo = fminf(tlo, t1);
+                    thi = fmaxf(thi, t1);
                     const float fd = (float)dlo;
                     const int la = __float2int_ru(fmaxf((tlo - r) - fd, 0.0f));
                     const int lb = __float2int_rd(fminf((thi + r) - fd, (float)(a.wd - 1)));
                     uint32_t ra = rst_a + (uint32_t)vl * rstv + (uint32_t)la * 32u;
                     uint32_t ya = yv + (uint32_t)la * PITCH;
                     for (int dl = la; dl <= lb; ++dl, ra += 32u, ya += PITCH) {
-                        const float4 A = lds4(ra), Bc = lds4(ra + 16);
-                        const float s0 = fmaf(px, Bc.x, fmaf(py0, Bc.y, Bc.z));
+                        const float4 A = lds4(ra);
+                        const float bx = A.z * a.ih2, by = A.w * a.ih2;   // as re-basing computed them
+                        const float s0 = fmaf(px, bx, fmaf(py0, by, lds1(ra + 16)));
                         float w[PX];
                         w[0] = bwdp_weight<KW>(px, py0, s0, A);
-                        if constexpr (PX == 2) w[1] = bwdp_weight<KW>(px, py0 + 1.0f, s0 + Bc.y, A);
+                        w[1] = bwdp_weight<KW>(px, py0 + 1.0f, s0 + by, A);
 #pragma unroll
                         for (int q = 0; q < NQ; ++q) {
                             const float4 y4 = lds4(ya + 16 * q);
-                            if constexpr (PX == 2) {
-                                // pixel pairs: paired FMAs (the same bits as scalar ones; measured 2-3 %
-                                // faster here, while the 32-image groups' single pixels ran slower paired)
+                            if constexpr (BG <= 16) {
+                                // paired FMAs (the same bits as scalar ones): half the instructions, which 8- and
+                                // 16-image groups issue among as many weights (2-3 % faster); 32-image groups
+                                // measured the same either way and spilled when paired
                                 const f32x2 y01 = f2_pack(y4.x, y4.y), y23 = f2_pack(y4.z, y4.w);
 #pragma unroll
                                 for (int x = 0; x < PX; ++x) {
@@ -700,7 +698,7 @@ radon_status launch_backward_packed_t(const radon_geometry* g, const void* packe
         return RADON_ERR_UNSUPPORTED;
     }
     // the geometry's weight table serves the exact adjoint's pixel pairs (16-bit or smaller groups)
-    const bool tab = kw > 0 && BwdPShape<BG>::PX == 2 && g->d_tab_w != nullptr && g->tab_kw == kw && g->tab_wd == wd;
+    const bool tab = kw > 0 && BG <= 16 && g->d_tab_w != nullptr && g->tab_kw == kw && g->tab_wd == wd;
     int stages = 2;
     // the table kernel stages ray rows too (for the pairs its table marks as overflowing)
     const size_t smem = bwdp_plan<T, BG>(wd, kw > 0, &stages);
@@ -742,7 +740,7 @@ radon_status launch_backward_packed_t(const radon_geometry* g, const void* packe
     a.tab_la = g->d_tab_la;
     const dim3 grid((unsigned)(a.tiles_x * a.tiles_x), (unsigned)groups);
     cudaError_t e;
-    if constexpr (BwdPShape<BG>::PX == 2) {
+    if constexpr (BG <= 16) {
         if (tab) {
             e = kw == 3 ? bwdp_launch<T, BG, 3, true>(map, rmap, a, grid, smem, s)
                         : bwdp_launch<T, BG, 6, true>(map, rmap, a, grid, smem, s);

@@ -146,4 +146,8 @@ __device__ __forceinline__ void sts4(uint32_t a, float4 v) {
                  : "memory");
 }
 
+__device__ __forceinline__ void sts1(uint32_t a, float v) {
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+
 }  // namespace radon
