@@ -415,12 +415,13 @@ def run_ours(args):
                 traffic_tab = json.load(f).get(args.workload, {}).get(args.storage, {})
         except (OSError, ValueError):
             traffic_tab = {}
-    # the gather-ceiling probe over as many texel groups per sample as the chosen forward's CTAs take
+    # the gather-ceiling probe over as many texel groups per sample as the chosen forward's CTAs take (two at
+    # most: CTAs of four groups go by texel rows, for which there is no probe)
     probe = ctypes.c_double(0.0)
     dt_code = {"f32": L.RADON_F32, "f16": L.RADON_F16, "bf16": L.RADON_BF16}[args.storage]
     bg = 4 if args.storage == "f32" else 8
     fwd_groups = max(1, forward_images_per_cta(geom, dt, B, chosen) // bg)
-    L.check(L.radon_probe_gather_ceiling_groups(dt_code, 0, fwd_groups, ctypes.byref(probe)),
+    L.check(L.radon_probe_gather_ceiling_groups(dt_code, 0, min(fwd_groups, 2), ctypes.byref(probe)),
             "radon_probe_gather_ceiling_groups")
     rooflines = {
         # forward: 4 texels per sample through the shared-memory / L1 load pipe, 128 B/clk/SM

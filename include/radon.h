@@ -240,9 +240,10 @@ RADON_API size_t radon_forward_workspace_size(const radon_geometry* geometry, ra
 
 /*
  * Images per CTA of the packed forward that radon_forward_ws (with a large enough workspace) runs for
- * this call: one texel group (8 for 16-bit storage, 4 for FP32) or two groups whose images share each
- * sample's position, floor and weight evaluation (16 / 8).  By default 16-bit batches of more than 8
- * images take two groups and FP32 one; `config`'s images_per_cta chooses where it holds one of those
+ * this call: one texel group (8 for 16-bit storage, 4 for FP32), two groups whose images share each
+ * sample's position, floor and weight evaluation (16 / 8), or four that share each texel row's weights (32
+ * / 16).  By default 16-bit batches of more than 8 images take two groups and of more than 24 four (FP32
+ * weights), FP32 batches of more than 16 images four and smaller ones one, where the bands fit; `config`'s images_per_cta chooses where it holds one of those
  * values.  Where no shape with one thread per ray fits a TMA box (sparse views with a detector wider
  * than the image) and `config` fixes no views per CTA, two threads share each ray (half the detectors
  * per CTA, one texel group).  *images = 0 when another kernel serves the call (one image under AUTO,

@@ -163,6 +163,8 @@ template <typename T, int MODE>
 cudaError_t launch_packed_t(const CUtensorMap& mr, const CUtensorMap& mc, const FwdTiledArgs& a, dim3 grid,
                             size_t smem, int NG, int LN, cudaStream_t s) {
     if (LN == 2) return launch_packed_ng<T, MODE, 1, 2>(mr, mc, a, grid, smem, s);
+    if constexpr (MODE == kMathScalar)
+        if (NG == 4) return launch_packed_ng<T, MODE, 4, 1>(mr, mc, a, grid, smem, s);
     return NG == 2 ? launch_packed_ng<T, MODE, 2, 1>(mr, mc, a, grid, smem, s)
                    : launch_packed_ng<T, MODE, 1, 1>(mr, mc, a, grid, smem, s);
 }
@@ -199,23 +201,41 @@ radon_status packed_forward_shape(radon_geometry* g, radon_dtype dt, int batch, 
     // texels (4 images each) measured slower paired.  Rows per slab: 16 for one group; 14 for two
     // (2 CTAs/SM), 8 with FP16 weights (3 CTAs/SM), the fastest of 8-16 rows measured.  A default pair
     // whose buffers would not fit falls back to one group.
-    int NG = lanes == 2 ? 1 : ipc != 0 ? (ipc == 2 * BG ? 2 : 1) : (esz == 2 && batch > BG ? 2 : 1);
+    // Four groups, row by row, where the batch fills most of one more CTA: 16-bit batches of more than
+    // 24 images (parallel 32 x 512^2, 512 views: FP16 1.78 -> 1.45 ms, BF16 1.55 -> 1.34; three groups cost
+    // about what a pair and a single do) and FP32 batches of more than 16 (2.33 -> 1.56 ms; 32 x 256^2, 256
+    // views 376 -> 242 us; smaller FP32 batches keep the one group that the query reports for them), in
+    // the highest slab of 8, 6 or 4 rows that leaves two CTAs per SM (8 rows 1.45 ms, 6 1.48, 4 1.56; 10
+    // rows at one CTA 1.88).  FP16 weights keep two groups.
+    int NG = lanes == 2 ? 1
+             : ipc != 0 ? (ipc == 2 * BG ? 2 : 1)
+             : !f16w && batch > (esz == 2 ? 24 : 16) ? 4
+                                                     : (esz == 2 && batch > BG ? 2 : 1);
+    const int fixed_rows = cfg ? cfg->rows_per_slab : 0;
+    int R = fixed_rows ? fixed_rows : 8;   // of four groups, lowered until they fit
     for (;;) {
-        const int R = cfg && cfg->rows_per_slab ? cfg->rows_per_slab : (NG == 2 ? (f16w ? 8 : 14) : 16);
+        if (NG != 4) R = fixed_rows ? fixed_rows : (NG == 2 ? (f16w ? 8 : 14) : 16);
         if (R < 2 || R > 64 || (R & 1)) {
             *why = "rows_per_slab must be even and in [2, 64]";
             return RADON_ERR_UNSUPPORTED;
         }
         const int maxw = forward_band_width(g, G, Dt, R);
         const int wbox = (maxw + 2 + 7) / 8 * 8;   // row pitch = 0 (mod 8) texels: fewest bank conflicts (measured)
+        // As many ring stages (up to 4) as keep three CTAs resident per SM (3 x (smem + 1 KB) <= 228 KB), two
+        // of four groups.
+        const size_t room = (NG == 4 ? 113 : 75) * 1024;
+        int stages = 2;
+        while (stages < kFwdMaxStages && fwd_packed_smem_bytes(R, wbox, stages + 1, NG) <= room) ++stages;
+        const size_t smem = fwd_packed_smem_bytes(R, wbox, stages, NG);
+        if (NG == 4 && (wbox > 256 || smem > room)) {
+            if (!fixed_rows && R > 4) R -= 2;
+            else NG = esz == 2 ? 2 : 1;
+            continue;
+        }
         if (wbox > 256) {
             *why = "working band wider than a TMA box";
             return RADON_ERR_UNSUPPORTED;
         }
-        // As many ring stages (up to 4) as keep three CTAs resident per SM (3 x (smem + 1 KB) <= 228 KB).
-        int stages = 2;
-        while (stages < kFwdMaxStages && fwd_packed_smem_bytes(R, wbox, stages + 1, NG) <= 75 * 1024) ++stages;
-        const size_t smem = fwd_packed_smem_bytes(R, wbox, stages, NG);
         if (smem <= 227 * 1024) {
             *out = PackedFwdShape{G, Dt, NG, lanes, R, wbox, stages, smem};
             return RADON_OK;
