@@ -199,16 +199,38 @@ radon_status validate_epilogue(const radon_epilogue* e, radon_dtype dt) {
 
 }  // namespace
 
-// The packed forward's config for shape candidate i (views per CTA 8, 4, 2, 1 in order unless the caller
-// fixed them); images per CTA: one texel group or two (a value meant for the adjoint leaves the default).
-radon_launch_config packed_forward_config(const radon_launch_config* cfg, radon_dtype dt, int i) {
-    static const int kViewsPacked[4] = {8, 4, 2, 1};
-    const bool fixed = cfg != nullptr && cfg->views_per_cta != 0;
+// The packed forward's config with `views` views per CTA; images per CTA: one texel group or two (a value
+// meant for the adjoint leaves the default).
+radon_launch_config packed_forward_config(const radon_launch_config* cfg, radon_dtype dt, int views) {
     const int bg = dt == RADON_F32 ? 4 : 8;
     const int ipc = cfg != nullptr && (cfg->images_per_cta == bg || cfg->images_per_cta == 2 * bg)
                         ? cfg->images_per_cta : 0;
-    return radon_launch_config{RADON_ALGO_TILED, fixed ? cfg->views_per_cta : kViewsPacked[i],
-                               cfg ? cfg->rows_per_slab : 0, ipc, 0, 0, cfg ? cfg->weights : 0};
+    return radon_launch_config{RADON_ALGO_TILED, views, cfg ? cfg->rows_per_slab : 0, ipc, 0, 0, cfg ? cfg->weights : 0};
+}
+
+int packed_forward_tries(radon_geometry* g, radon_dtype dt, int batch, const radon_launch_config* cfg, bool f16w,
+                         PackedTry* out) {
+    if (cfg != nullptr && cfg->views_per_cta != 0) {
+        out[0] = PackedTry{cfg->views_per_cta, 1};
+        return 1;
+    }
+    int n = 0;
+    const int bg = dt == RADON_F32 ? 4 : 8;
+    const radon_launch_config c8 = packed_forward_config(cfg, dt, 8);
+    PackedFwdShape sh;
+    std::string why;
+    if (batch <= bg && c8.images_per_cta != 2 * bg &&
+        packed_forward_shape(g, dt, batch, &c8, f16w, 1, &sh, &why) == RADON_OK) {
+        // One texel group on fewer than two CTAs per SM: each warp waits for its own loads, and twice the warps
+        // over bands of half the views are faster (8 x 512^2 BF16, 60 views, 184 CTAs: 127 -> 104 us; 368
+        // CTAs of 120 views: 178 against 183).  FP32 bands take twice the copies per image: only where
+        // not even one CTA per SM runs (4 x 128^2, 128 views, 96 CTAs: 33 -> 28 us; 184 CTAs: 157 against 174).
+        const long long ctas = (long long)g->group_count[3] * ((g->D + sh.Dt - 1) / sh.Dt);
+        if (ctas < (dt == RADON_F32 ? 152 : 2 * 152)) out[n++] = PackedTry{4, 2};
+    }
+    for (int lanes = 1; lanes <= 2; ++lanes)
+        for (int views = 8; views >= 1; views /= 2) out[n++] = PackedTry{views, lanes};
+    return n;
 }
 
 // One image under AUTO with no tile parameters runs the single-image kernels.
@@ -288,29 +310,24 @@ radon_status project(const radon_geometry* g, const void* in, void* out, radon_d
     }
     if (forward && algo != RADON_ALGO_PLAIN && ws != nullptr && ws_bytes >= packed_image_bytes(g->n, batch, dt)) {
         // Packed path: pack the batch once, then copy bands of texels straight into shared memory.
-        // one lane per ray first; where no one-lane shape fits and the caller left the shape to the
-        // library, two lanes (half the detectors per CTA: narrower bands).  An explicit views per
-        // CTA keeps one lane per ray.
-        const bool fixed = cfg != nullptr && cfg->views_per_cta != 0;
+        const bool f16w = dt == RADON_F16 && cfg != nullptr && cfg->weights == RADON_WEIGHTS_F16 && ep.add == nullptr;
+        PackedTry tries[kMaxPackedTries];
+        const int n_tries = packed_forward_tries(const_cast<radon_geometry*>(g), dt, batch, cfg, f16w, tries);
         std::string why;
-        bool packed_done = false;
-        for (int lanes = 1; lanes <= (fixed ? 1 : 2); ++lanes) {
-            for (int i = 0; i < (fixed ? 1 : 4); ++i) {
-                const radon_launch_config c = packed_forward_config(cfg, dt, i);
-                if (!packed_done) {
-                    cudaError_t e = launch_pack_images(in, ws, g->n, batch, dt, s);
-                    if (e != cudaSuccess) return cuda_fail(e, "pack launch");
-                    count_launches(1);
-                    packed_done = true;
-                }
-                st = launch_forward_packed(const_cast<radon_geometry*>(g), ws, out, dt, batch, &c, ep, s, &why,
-                                           lanes);
-                if (st == RADON_OK) {
-                    count_launches(1);
-                    return RADON_OK;
-                }
-                if (st != RADON_ERR_UNSUPPORTED) return fail(st, why);
+        for (int i = 0; i < n_tries; ++i) {
+            const radon_launch_config c = packed_forward_config(cfg, dt, tries[i].views);
+            if (i == 0) {
+                cudaError_t e = launch_pack_images(in, ws, g->n, batch, dt, s);
+                if (e != cudaSuccess) return cuda_fail(e, "pack launch");
+                count_launches(1);
             }
+            st = launch_forward_packed(const_cast<radon_geometry*>(g), ws, out, dt, batch, &c, ep, s, &why,
+                                       tries[i].lanes);
+            if (st == RADON_OK) {
+                count_launches(1);
+                return RADON_OK;
+            }
+            if (st != RADON_ERR_UNSUPPORTED) return fail(st, why);
         }
         // no packed shape fits: continue with the paths that need no workspace
     }
@@ -493,17 +510,16 @@ radon_status radon_forward_images_per_cta(const radon_geometry* g, radon_dtype d
     const int algo = config ? config->algo : RADON_ALGO_AUTO;
     if (batch == 0 || algo == RADON_ALGO_PLAIN || single_image_call(config, batch)) return RADON_OK;
     const bool f16w = dtype == RADON_F16 && config != nullptr && config->weights == RADON_WEIGHTS_F16;
-    const bool fixed = config != nullptr && config->views_per_cta != 0;
-    for (int lanes = 1; lanes <= (fixed ? 1 : 2); ++lanes) {
-        for (int i = 0; i < (fixed ? 1 : 4); ++i) {
-            const radon_launch_config c = packed_forward_config(config, dtype, i);
-            PackedFwdShape sh;
-            std::string why;
-            if (packed_forward_shape(const_cast<radon_geometry*>(g), dtype, batch, &c, f16w, lanes, &sh, &why) ==
-                RADON_OK) {
-                *images = sh.NG * (dtype == RADON_F32 ? 4 : 8);
-                return RADON_OK;
-            }
+    PackedTry tries[kMaxPackedTries];
+    const int n_tries = packed_forward_tries(const_cast<radon_geometry*>(g), dtype, batch, config, f16w, tries);
+    for (int i = 0; i < n_tries; ++i) {
+        const radon_launch_config c = packed_forward_config(config, dtype, tries[i].views);
+        PackedFwdShape sh;
+        std::string why;
+        if (packed_forward_shape(const_cast<radon_geometry*>(g), dtype, batch, &c, f16w, tries[i].lanes, &sh, &why) ==
+            RADON_OK) {
+            *images = sh.NG * (dtype == RADON_F32 ? 4 : 8);
+            return RADON_OK;
         }
     }
     return RADON_OK;
