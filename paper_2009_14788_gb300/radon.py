@@ -17,6 +17,22 @@ import torch
 
 from . import _lib as L
 
+# The current stream's handle without building a torch.cuda.Stream around it (a fifth of the time), where
+# this torch has it.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or \
+    (lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
+def _call(fn, device, *args) -> int:
+    """The library call ``fn(*args, stream)`` on ``device``'s current stream with ``device`` current; the
+    device is switched only where another one is (a switch and back costs as much as the call)."""
+    index = device.index
+    if torch.cuda.current_device() == index:
+        return fn(*args, _raw_stream(index))
+    with torch.cuda.device(index):
+        return fn(*args, _raw_stream(index))
+
+
 _DTYPES = {torch.float32: L.RADON_F32, torch.float16: L.RADON_F16, torch.bfloat16: L.RADON_BF16}
 
 ALGOS = {"auto": L.RADON_ALGO_AUTO, "plain": L.RADON_ALGO_PLAIN, "tiled": L.RADON_ALGO_TILED}
@@ -73,6 +89,10 @@ class Geometry:
     @property
     def handle(self):
         return self._h
+
+    @property
+    def lib(self):
+        return self._lib
 
     @property
     def angles(self) -> np.ndarray:
@@ -155,7 +175,7 @@ def _check_out(out: torch.Tensor, like: torch.Tensor, shape) -> torch.Tensor:
 
 def forward_workspace_bytes(geom: Geometry, dtype: torch.dtype, batch: int) -> int:
     """Bytes of the workspace the packed forward path uses (``radon_forward_workspace_size``)."""
-    return int(L.radon_forward_workspace_size(geom.handle, _DTYPES[dtype], int(batch)))
+    return geom.lib.radon_forward_workspace_size(geom.handle, _DTYPES[dtype], batch)
 
 
 def forward_images_per_cta(geom: Geometry, dtype: torch.dtype, batch: int, config=None) -> int:
@@ -181,7 +201,6 @@ def forward_raw(geom: Geometry, x: torch.Tensor, config=None, out=None, workspac
     batch = x.numel() // (geom.n * geom.n)
     shape = tuple(x.shape[:-2]) + geom.sino_shape
     y = torch.empty(shape, dtype=x.dtype, device=x.device) if out is None else _check_out(out, x, shape)
-    stream = torch.cuda.current_stream(x.device).cuda_stream
     ws_ptr, ws_bytes = None, 0
     if isinstance(workspace, str) and workspace == "auto":
         need = forward_workspace_bytes(geom, x.dtype, batch)
@@ -193,22 +212,21 @@ def forward_raw(geom: Geometry, x: torch.Tensor, config=None, out=None, workspac
         if workspace.device != x.device or not workspace.is_contiguous():
             raise ValueError("workspace must be a contiguous tensor on %s" % x.device)
         ws_ptr, ws_bytes = workspace.data_ptr(), workspace.numel() * workspace.element_size()
-    with torch.cuda.device(x.device):
-        cfg = ctypes.byref(config) if config is not None else None
-        if ws_ptr is not None:
-            st = L.radon_forward_ws(geom.handle, x.data_ptr(), y.data_ptr(), _DTYPES[x.dtype], batch, cfg, ws_ptr,
-                                    ws_bytes, stream)
-        elif config is None:
-            st = L.radon_forward(geom.handle, x.data_ptr(), y.data_ptr(), _DTYPES[x.dtype], batch, stream)
-        else:
-            st = L.radon_forward_ex(geom.handle, x.data_ptr(), y.data_ptr(), _DTYPES[x.dtype], batch, cfg, stream)
+    cfg = ctypes.byref(config) if config is not None else None
+    head = (geom.handle, x.data_ptr(), y.data_ptr(), _DTYPES[x.dtype], batch)
+    if ws_ptr is not None:
+        st = _call(geom.lib.radon_forward_ws, x.device, *head, cfg, ws_ptr, ws_bytes)
+    elif config is None:
+        st = _call(geom.lib.radon_forward, x.device, *head)
+    else:
+        st = _call(geom.lib.radon_forward_ex, x.device, *head, cfg)
     L.check(st, "radon_forward")
     return y
 
 
 def backward_workspace_bytes(geom: Geometry, dtype: torch.dtype, batch: int) -> int:
     """Bytes of the workspace the packed adjoint path uses (``radon_backward_workspace_size``)."""
-    return int(L.radon_backward_workspace_size(geom.handle, _DTYPES[dtype], int(batch)))
+    return geom.lib.radon_backward_workspace_size(geom.handle, _DTYPES[dtype], batch)
 
 
 def _workspace(workspace, need, device):
@@ -230,17 +248,15 @@ def backward_raw(geom: Geometry, y: torch.Tensor, config=None, out=None, workspa
     batch = y.numel() // (geom.n_angles * geom.det_count)
     shape = tuple(y.shape[:-2]) + (geom.n, geom.n)
     x = torch.empty(shape, dtype=y.dtype, device=y.device) if out is None else _check_out(out, y, shape)
-    stream = torch.cuda.current_stream(y.device).cuda_stream
     ws = _workspace(workspace, backward_workspace_bytes(geom, y.dtype, batch) if batch > 0 else 0, y.device)
-    with torch.cuda.device(y.device):
-        cfg = ctypes.byref(config) if config is not None else None
-        if ws is not None:
-            st = L.radon_backward_ws(geom.handle, y.data_ptr(), x.data_ptr(), _DTYPES[y.dtype], batch, cfg,
-                                     ws.data_ptr(), ws.numel() * ws.element_size(), stream)
-        elif config is None:
-            st = L.radon_backward(geom.handle, y.data_ptr(), x.data_ptr(), _DTYPES[y.dtype], batch, stream)
-        else:
-            st = L.radon_backward_ex(geom.handle, y.data_ptr(), x.data_ptr(), _DTYPES[y.dtype], batch, cfg, stream)
+    cfg = ctypes.byref(config) if config is not None else None
+    head = (geom.handle, y.data_ptr(), x.data_ptr(), _DTYPES[y.dtype], batch)
+    if ws is not None:
+        st = _call(geom.lib.radon_backward_ws, y.device, *head, cfg, ws.data_ptr(), ws.numel() * ws.element_size())
+    elif config is None:
+        st = _call(geom.lib.radon_backward, y.device, *head)
+    else:
+        st = _call(geom.lib.radon_backward_ex, y.device, *head, cfg)
     L.check(st, "radon_backward")
     return x
 
@@ -271,12 +287,9 @@ def forward_fused(geom: Geometry, x: torch.Tensor, op_scale=1.0, op_scale_dev=No
         raise ValueError("add must have shape %s" % (shape,))
     ep = _epilogue(op_scale, op_scale_dev, add_scale, add, y)
     ws = _workspace(workspace, forward_workspace_bytes(geom, x.dtype, batch) if batch > 0 else 0, x.device)
-    stream = torch.cuda.current_stream(x.device).cuda_stream
-    with torch.cuda.device(x.device):
-        st = L.radon_forward_fused(geom.handle, x.data_ptr(), y.data_ptr(), _DTYPES[x.dtype], batch, ctypes.byref(ep),
-                                   ctypes.byref(config) if config is not None else None,
-                                   ws.data_ptr() if ws is not None else None,
-                                   ws.numel() if ws is not None else 0, stream)
+    st = _call(geom.lib.radon_forward_fused, x.device, geom.handle, x.data_ptr(), y.data_ptr(), _DTYPES[x.dtype], batch,
+               ctypes.byref(ep), ctypes.byref(config) if config is not None else None,
+               ws.data_ptr() if ws is not None else None, ws.numel() if ws is not None else 0)
     L.check(st, "radon_forward_fused")
     return y
 
@@ -295,12 +308,9 @@ def backward_fused(geom: Geometry, y: torch.Tensor, op_scale=1.0, op_scale_dev=N
         raise ValueError("add must have shape %s" % (shape,))
     ep = _epilogue(op_scale, op_scale_dev, add_scale, add, x)
     ws = _workspace(workspace, backward_workspace_bytes(geom, y.dtype, batch) if batch > 0 else 0, y.device)
-    stream = torch.cuda.current_stream(y.device).cuda_stream
-    with torch.cuda.device(y.device):
-        st = L.radon_backward_fused(geom.handle, y.data_ptr(), x.data_ptr(), _DTYPES[y.dtype], batch, ctypes.byref(ep),
-                                    ctypes.byref(config) if config is not None else None,
-                                    ws.data_ptr() if ws is not None else None,
-                                    ws.numel() if ws is not None else 0, stream)
+    st = _call(geom.lib.radon_backward_fused, y.device, geom.handle, y.data_ptr(), x.data_ptr(), _DTYPES[y.dtype], batch,
+               ctypes.byref(ep), ctypes.byref(config) if config is not None else None,
+               ws.data_ptr() if ws is not None else None, ws.numel() if ws is not None else 0)
     L.check(st, "radon_backward_fused")
     return x
 
@@ -393,10 +403,8 @@ def filter_sinogram(geom: Geometry, y: torch.Tensor, filter_name: str = "ram-lak
     y = y.contiguous()
     batch = y.numel() // (geom.n_angles * geom.det_count)
     q = torch.empty_like(y) if out is None else _check_out(out, y, tuple(y.shape))
-    stream = torch.cuda.current_stream(y.device).cuda_stream
-    with torch.cuda.device(y.device):
-        st = L.radon_filter_sinogram(geom.handle, y.data_ptr(), q.data_ptr(), _DTYPES[y.dtype], batch,
-                                     L.FILTERS[filter_name], stream)
+    st = _call(geom.lib.radon_filter_sinogram, y.device, geom.handle, y.data_ptr(), q.data_ptr(), _DTYPES[y.dtype],
+               batch, L.FILTERS[filter_name])
     L.check(st, "radon_filter_sinogram")
     return q
 
