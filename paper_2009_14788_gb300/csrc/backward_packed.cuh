@@ -231,62 +231,73 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
 
     if (tid >= NC) {
         // ------------------------------------------------------------------ producer warp
+        // One lane prepares one view, 32 views (eight chunks) at a time: a window takes two dozen divisions
+        // and a trip to L2, which four lanes at a time left as the longest chain of a chunk.
         const int lane = tid & 31;
         int c = 0;
-        for (; c < nchunks; ++c) {
-            const int st = c % S;
-            bool ok = true;
-            if (c >= S && lane == 0) ok = mbar_wait_bounded(&empty[st], (uint32_t)((c / S - 1) & 1), a.spin_limit);
-            if (!__shfl_sync(0xffffffffu, ok ? 1 : 0, 0)) break;
-            const int v0 = c * kBwdPViews;
-            const int nv = min(kBwdPViews, a.V - v0);
-            if (lane < nv) {
-                const ViewF vf = a.views[v0 + lane];
-                int dlo;
-                float r;
+        bool ok = true;
+        while (ok && c < nchunks) {
+            const int vlane = c * kBwdPViews + lane;
+            ViewF vf{};
+            int dlo = 0;
+            float r = 0.0f;
+            unsigned flagged = 0;
+            if (vlane < a.V) {
+                vf = a.views[vlane];
                 bwd_view_window(vf, ti, tj, a.n, &dlo, &r);
                 // every pixel's candidates [ceil(t - r), floor(t + r)] within the detector must lie in
                 // the copied window; the consumers clamp to it, so a miss is recorded, not overrun
                 const float thi = floorf(bwdp_tile_tmax(vf, ti, tj, a.n) + r);
                 if (fminf(thi, (float)(a.D - 1)) > (float)(dlo + a.wd - 1)) record_device_error(a.err, RADON_ERR_DEVICE_BOUNDS);
-                dlo_c[st * kBwdPViews + lane] = dlo;
-                r_c[st * kBwdPViews + lane] = r;
-                view_c[st * kBwdPViews + lane] = vf;
             }
             // ray rows: always for the on-the-fly weights; with a table only where some pair overflows
-            bool rays = kRays;
             if constexpr (TAB) {
-                const int fl = lane < nv ? __ldg(a.tab_vflag + (size_t)tile * a.V + v0 + lane) : 0;
-                rays = __any_sync(0xffffffffu, fl != 0);
+                const int fl = vlane < a.V ? __ldg(a.tab_vflag + (size_t)tile * a.V + vlane) : 0;
+                flagged = __ballot_sync(0xffffffffu, fl != 0);
             }
-            __syncwarp();
-            if (lane == 0) {
-                unsigned char* slot = ring + (size_t)st * m.stage;
-                rays_c[st] = rays ? 1 : 0;
-                fence_proxy_async_shared();
-                mbar_arrive_expect_tx(&tma_bar[st],
-                                      (uint32_t)(nv * a.wd * (L::kRowElems * (int)sizeof(T) + (rays ? 32 : 0))));
-                for (int vl = 0; vl < nv; ++vl) {
-                    const int dlo = dlo_c[st * kBwdPViews + vl];
-                    tma_load_4d(slot + (size_t)vl * m.yst_view, &map, &tma_bar[st], 0, dlo, v0 + vl, blockIdx.y);
-                    if (rays)   // the interpolating backprojector needs no rays
-                        tma_load_2d(slot + (size_t)kBwdPViews * m.yst_view + (size_t)vl * m.rst_view, &rmap,
-                                    &tma_bar[st], 0, (v0 + vl) * a.D + dlo);
+            for (int k = 0; k < 32 / kBwdPViews && c < nchunks; ++k, ++c) {
+                const int st = c % S;
+                if (c >= S && lane == 0) ok = mbar_wait_bounded(&empty[st], (uint32_t)((c / S - 1) & 1), a.spin_limit);
+                ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                if (!ok) break;
+                const int v0 = c * kBwdPViews;
+                const int nv = min(kBwdPViews, a.V - v0);
+                if (lane / kBwdPViews == k && vlane < a.V) {
+                    const int w = st * kBwdPViews + lane % kBwdPViews;
+                    dlo_c[w] = dlo;
+                    r_c[w] = r;
+                    view_c[w] = vf;
                 }
-                if constexpr (TAB) {
-                    // the table rows of the chunk that will next use this slot, into L2 (a hint: no
-                    // completion to wait for); 16-byte aligned multiples of 16 bytes by construction
-                    const int cn = c + S;
-                    if (cn < nchunks) {
-                        const int vn = cn * kBwdPViews, nvn = min(kBwdPViews, a.V - vn);
-                        const size_t rec = ((size_t)tile * a.V + vn) * kBwdTabPairs;
-                        bulk_prefetch_l2(a.tab_w + 2 * rec, (uint32_t)(nvn * kBwdTabPairs * 32));
-                        bulk_prefetch_l2(a.tab_w5 + rec, (uint32_t)(nvn * kBwdTabPairs * 8));
-                        bulk_prefetch_l2(a.tab_la + rec, (uint32_t)(nvn * kBwdTabPairs * 4));
+                const bool rays = kRays && (!TAB || ((flagged >> (k * kBwdPViews)) & ((1u << kBwdPViews) - 1u)) != 0);
+                __syncwarp();
+                if (lane == 0) {
+                    unsigned char* slot = ring + (size_t)st * m.stage;
+                    rays_c[st] = rays ? 1 : 0;
+                    fence_proxy_async_shared();
+                    mbar_arrive_expect_tx(&tma_bar[st],
+                                          (uint32_t)(nv * a.wd * (L::kRowElems * (int)sizeof(T) + (rays ? 32 : 0))));
+                    for (int vl = 0; vl < nv; ++vl) {
+                        const int d0 = dlo_c[st * kBwdPViews + vl];
+                        tma_load_4d(slot + (size_t)vl * m.yst_view, &map, &tma_bar[st], 0, d0, v0 + vl, blockIdx.y);
+                        if (rays)   // the interpolating backprojector needs no rays
+                            tma_load_2d(slot + (size_t)kBwdPViews * m.yst_view + (size_t)vl * m.rst_view, &rmap,
+                                        &tma_bar[st], 0, (v0 + vl) * a.D + d0);
+                    }
+                    if constexpr (TAB) {
+                        // the table rows of the chunk that will next use this slot, into L2 (a hint: no
+                        // completion to wait for); 16-byte aligned multiples of 16 bytes by construction
+                        const int cn = c + S;
+                        if (cn < nchunks) {
+                            const int vn = cn * kBwdPViews, nvn = min(kBwdPViews, a.V - vn);
+                            const size_t rec = ((size_t)tile * a.V + vn) * kBwdTabPairs;
+                            bulk_prefetch_l2(a.tab_w + 2 * rec, (uint32_t)(nvn * kBwdTabPairs * 32));
+                            bulk_prefetch_l2(a.tab_w5 + rec, (uint32_t)(nvn * kBwdTabPairs * 8));
+                            bulk_prefetch_l2(a.tab_la + rec, (uint32_t)(nvn * kBwdTabPairs * 4));
+                        }
                     }
                 }
+                __syncwarp();
             }
-            __syncwarp();
         }
         if (c < nchunks && lane == 0) {
             // The consumers stopped releasing slots: record it, let the copies still in flight land
