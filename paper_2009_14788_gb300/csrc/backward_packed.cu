@@ -52,12 +52,11 @@ int backward_packed_images_per_cta(const radon_geometry* g, int batch, radon_dty
     if (cfg != nullptr && cfg->images_per_cta != 0) return cfg->images_per_cta;
     if (batch <= 8) return 8;
     if (batch <= 16) return 16;
-    // with the geometry's weight table 16-bit 16-image groups read their weights, which measured faster
-    // than 32-image groups computing them (parallel 32 x 512^2, 512 views, FP16 adjoint: 1.84 vs 1.94
-    // ms; FP32 rows measured no faster: a step of 4.32 vs 4.27 ms)
-    if (g->d_tab_w != nullptr && dt != RADON_F32) return 16;
-    // A 32-image CTA costs about 1.56x a 16-image one (1.38x on parallel 512^2 with 512 views, 1.6x on
-    // 360-view fans with 1024 detectors): take it when its groups cost less and its staging fits one CTA's
+    // with a fan's weight table 16-bit 16-image groups read their weights, which measured faster than 32-image
+    // groups computing them
+    if (g->fan && bwdp_table_serves(g, 16) && dt != RADON_F32) return 16;
+    // A 32-image CTA costs about 1.56x a 16-image one (1.36-1.51x on parallel 512^2 with 512 views, 1.6x
+    // on 360-view fans with 1024 detectors): take it when its groups cost less and its staging fits one CTA's
     // shared memory.
     const long long g32 = (batch + 31) / 32, g16 = (batch + 15) / 16;
     if (25 * g32 < 16 * g16 && smem_32(g, dt) <= 227 * 1024) return 32;
@@ -171,12 +170,10 @@ radon_status build_adjoint_table(radon_geometry* g, std::string* why) {
     if (e == cudaSuccess) {
         const dim3 grid((unsigned)(tiles_x * tiles_x), (unsigned)((g->V + kViewsPerBlock - 1) / kViewsPerBlock));
         const float ih2 = (float)(1.0 / (g->h * g->h));
-        if (kw == 3)
-            bwdp_table_kernel<3><<<grid, kBwdTabPairs>>>(g->d_ray, g->d_view, g->n, g->V, g->D, ih2, wd, tiles_x,
-                                                         kViewsPerBlock, w, w5, la, vflag, over);
-        else
-            bwdp_table_kernel<6><<<grid, kBwdTabPairs>>>(g->d_ray, g->d_view, g->n, g->V, g->D, ih2, wd, tiles_x,
-                                                         kViewsPerBlock, w, w5, la, vflag, over);
+        auto kern = g->fan ? (kw == 3 ? bwdp_table_kernel<3, false> : bwdp_table_kernel<6, false>)
+                           : (kw == 3 ? bwdp_table_kernel<3, true> : bwdp_table_kernel<6, true>);
+        kern<<<grid, kBwdTabPairs>>>(g->d_ray, g->d_view, g->n, g->V, g->D, ih2, wd, tiles_x, kViewsPerBlock, w, w5, la,
+                                     vflag, over);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaDeviceSynchronize();
     }

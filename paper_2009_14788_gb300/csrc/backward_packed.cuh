@@ -20,6 +20,7 @@
 #pragma once
 
 #include <string>
+#include <type_traits>
 
 #include "backward_tiled.cuh"
 #include "dtype.cuh"
@@ -82,6 +83,7 @@ __host__ __device__ inline BwdPSmem bwdp_smem(int wd, int stages, bool rays) {
 
 struct BwdPArgs {
     const ViewF* views;
+    const RayT* rays;  // the ray table (parallel beams)
     void* img;
     int n, V, D, B;
     float h;           // output scale (the step; 1 for the interpolating backprojector)
@@ -163,6 +165,99 @@ __device__ __forceinline__ float bwdp_weight(float px, float py, float s, const 
     return w;
 }
 
+// Parallel beams: every ray of a view has the same step and the rays' sample lattices line up (sample k of ray
+// d + 1 is sample k of ray d moved by det_spacing * n, n the detector axis), so one re-based ray per view and
+// tile places them all.  A view's record, for tile-local pixels p and window rays l = 0, 1, ...:
+//   t = ax px + ay py + a0               window-relative detector coordinate
+//   s = b . p + c, b = step / h^2        its nearest integer is the first candidate sample (the same
+//                                        lattice index on every ray; c holds the window's half width)
+//   A + k step + (l - l0) n - p          sample k of window ray l relative to the pixel, n = q (ax, ay)
+// The reference ray l0 is the one nearest the window's middle, so the error of n is multiplied little.  A
+// candidate ray then costs a pixel two additions and its samples' tents instead of a record's two shared
+// loads, its first sample and its offset from the pixel, and no ray rows are copied or re-based (us, ray
+// records -> one ray per view, FP32, 512 views of 512^2: 8 images 898 -> 675, 16 images 1056 -> 854, 32
+// images 1581 -> 1286; 4 x 64^2, 64 views: 42 -> 30).
+struct BwdPPar {
+    float ax, ay, a0, c;
+    float Ax, Ay, sx, sy;
+    float q, l0;
+};
+
+__device__ __forceinline__ BwdPPar bwdp_par_view(const ViewF vf, const RayT* __restrict__ rays, int v, int D, int wd,
+                                                 int dlo, int ti, int tj, float ih2) {
+    const int dref = min(max(dlo + (wd >> 1), 0), D - 1);
+    const float4 A = bwd_ray_pos_rec(rays[(long long)v * D + dref], true, ti, tj, ih2);
+    const float bx = A.z * ih2, by = A.w * ih2;
+    BwdPPar w;
+    w.ax = vf.ax;
+    w.ay = vf.ay;
+    w.a0 = bwd_det_coord(vf, (float)tj, (float)ti) - (float)dlo;
+    w.c = (-fmaf(A.x, bx, A.y * by) - fmaf(fabsf(A.z) + fabsf(A.w), ih2, 1e-4f)) + 0.5f;
+    w.Ax = A.x;
+    w.Ay = A.y;
+    w.sx = A.z;
+    w.sy = A.w;
+    w.q = 1.0f / fmaf(vf.ax, vf.ax, vf.ay * vf.ay);
+    w.l0 = (float)(dref - dlo);
+    return w;
+}
+
+// A pixel pair's walk over the window rays of one view: [la, lb] the union of the pixels' candidates,
+// (rx, ry) each pixel's first candidate sample on ray la, (nx, ny) the move to the next ray.
+struct BwdPWalk {
+    int la, lb;
+    float rx[2], ry[2], nx, ny;
+};
+
+__device__ __forceinline__ BwdPWalk bwdp_par_walk(const BwdPPar w, float r, float px, float py0, float ih2, int wd) {
+    constexpr float kMagic = 12582912.0f;   // 1.5 * 2^23: x + kMagic rounds x to the nearest integer
+    BwdPWalk k;
+    const float t0 = fmaf(w.ax, px, fmaf(w.ay, py0, w.a0)), t1 = t0 + w.ay;
+    const float fa = ceilf(fmaxf(fminf(t0, t1) - r, 0.0f));
+    k.la = (int)fa;
+    k.lb = __float2int_rd(fminf(fmaxf(t0, t1) + r, (float)(wd - 1)));
+    k.nx = w.ax * w.q;
+    k.ny = w.ay * w.q;
+    const float bx = w.sx * ih2, by = w.sy * ih2;
+    const float s0 = fmaf(bx, px, fmaf(by, py0, w.c));
+    const float ka0 = (s0 + kMagic) - kMagic, ka1 = ((s0 + by) + kMagic) - kMagic;
+    const float l = fa - w.l0;
+    const float ux = fmaf(l, k.nx, w.Ax - px), uy0 = fmaf(l, k.ny, w.Ay - py0), uy1 = fmaf(l, k.ny, w.Ay - (py0 + 1.0f));
+    k.rx[0] = fmaf(ka0, w.sx, ux);
+    k.ry[0] = fmaf(ka0, w.sy, uy0);
+    k.rx[1] = fmaf(ka1, w.sx, ux);
+    k.ry[1] = fmaf(ka1, w.sy, uy1);
+    return k;
+}
+
+// The sum over KW consecutive samples from (rx, ry) of tent(rx) * tent(ry) (see bwdp_weight); and the same bits
+// with the steps as f32x2 additions: fewer instructions for the same pipe.
+template <int KW>
+__device__ __forceinline__ float bwdp_tents(float rx, float ry, float sx, float sy) {
+    float w = __saturatef(1.0f - fabsf(rx)) * __saturatef(1.0f - fabsf(ry));
+#pragma unroll
+    for (int k = 1; k < KW; ++k) {
+        rx += sx;
+        ry += sy;
+        w = fmaf(__saturatef(1.0f - fabsf(rx)), __saturatef(1.0f - fabsf(ry)), w);
+    }
+    return w;
+}
+
+template <int KW>
+__device__ __forceinline__ float bwdp_tents2(f32x2 r, f32x2 step) {
+    float rx, ry;
+    f2_unpack(r, &rx, &ry);
+    float w = __saturatef(1.0f - fabsf(rx)) * __saturatef(1.0f - fabsf(ry));
+#pragma unroll
+    for (int k = 1; k < KW; ++k) {
+        r = f2_add(r, step);
+        f2_unpack(r, &rx, &ry);
+        w = fmaf(__saturatef(1.0f - fabsf(rx)), __saturatef(1.0f - fabsf(ry)), w);
+    }
+    return w;
+}
+
 // 16-bit row segment of 8 images (one 16-byte load) -> 8 FP32 words (two 16-byte stores).
 template <typename T>
 __device__ __forceinline__ void bwdp_widen8(const uint4 u, float4* out);
@@ -189,12 +284,14 @@ __device__ __forceinline__ void bwdp_widen8<__nv_bfloat16>(const uint4 u, float4
 // being evaluated from re-based ray records; ray rows are copied and re-based only for chunks with a
 // view in which some pair of the tile overflows the table (the table's per-view flags).  The producer
 // prefetches the table's rows for the chunk that will next reuse its ring slot into L2.
-template <typename T, int BG, int KW, bool TAB = false>
+template <typename T, int BG, int KW, bool TAB, bool PAR>
 __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasPerSm)
     backward_packed_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap rmap,
                            const BwdPArgs a) {
-    static_assert(!TAB || (KW > 0 && BG <= 16), "the weight table serves the exact adjoint's smaller groups");
-    constexpr bool kRays = KW > 0;   // ray rows copied and re-based per chunk
+    static_assert(!TAB || (KW > 0 && BG <= 16 && (!PAR || (BG == 16 && KW == 6))),
+                  "the weight table serves the exact adjoint's smaller groups where it is faster");
+    static_assert(!PAR || KW > 0, "the interpolating backprojector takes its views as they are");
+    constexpr bool kRays = KW > 0 && !PAR;   // ray rows copied and re-based per chunk
     using L = BwdPLayout<T, BG>;
     constexpr int NQ = BG / 4;
     constexpr int PITCH = L::kPitch;
@@ -208,8 +305,11 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
     int* dlo_c = reinterpret_cast<int*>(smem + 192);              // [stages][views]
     float* r_c = reinterpret_cast<float*>(smem + 256);            // [stages][views]
     ViewF* view_c = reinterpret_cast<ViewF*>(smem + 512);         // [stages][views]
-    int* rays_c = reinterpret_cast<int*>(smem + 320);             // [stages]: the chunk's ray rows were copied
-    static_assert(kBwdPMaxStages * kBwdPViews * 4 <= 64 && 512 + kBwdPMaxStages * kBwdPViews * 32 <= kBwdPHeader,
+    int* fly_c = reinterpret_cast<int*>(smem + 320);              // [stages]: the chunk takes weights on the fly
+    float2* par_c = reinterpret_cast<float2*>(smem + 352);        // [stages][views] parallel: (q, l0)
+    static_assert(kBwdPMaxStages * kBwdPViews * 4 <= 64 && kBwdPMaxStages * 4 <= 32 &&
+                      352 + kBwdPMaxStages * kBwdPViews * 8 <= 512 &&
+                      512 + kBwdPMaxStages * kBwdPViews * 32 <= kBwdPHeader && sizeof(ViewF) == 32,
                   "ring header overflows its slots");
     const int S = a.stages;
     const BwdPSmem m = bwdp_smem<T, BG>(a.wd, S, kRays);
@@ -239,6 +339,7 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
         while (ok && c < nchunks) {
             const int vlane = c * kBwdPViews + lane;
             ViewF vf{};
+            float2 par = make_float2(0.0f, 0.0f);
             int dlo = 0;
             float r = 0.0f;
             unsigned flagged = 0;
@@ -249,8 +350,20 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
                 // the copied window; the consumers clamp to it, so a miss is recorded, not overrun
                 const float thi = floorf(bwdp_tile_tmax(vf, ti, tj, a.n) + r);
                 if (fminf(thi, (float)(a.D - 1)) > (float)(dlo + a.wd - 1)) record_device_error(a.err, RADON_ERR_DEVICE_BOUNDS);
+                if constexpr (PAR) {   // the first eight words of the view's record in the place of its map
+                    const BwdPPar w = bwdp_par_view(vf, a.rays, vlane, a.D, a.wd, dlo, ti, tj, a.ih2);
+                    vf.ax = w.ax;
+                    vf.ay = w.ay;
+                    vf.a0 = w.a0;
+                    vf.bx = w.c;
+                    vf.by = w.Ax;
+                    vf.b0 = w.Ay;
+                    vf.major = __float_as_int(w.sx);
+                    vf.pad = __float_as_int(w.sy);
+                    par = make_float2(w.q, w.l0);
+                }
             }
-            // ray rows: always for the on-the-fly weights; with a table only where some pair overflows
+            // weights on the fly: always without a table, with one only where some pair overflows
             if constexpr (TAB) {
                 const int fl = vlane < a.V ? __ldg(a.tab_vflag + (size_t)tile * a.V + vlane) : 0;
                 flagged = __ballot_sync(0xffffffffu, fl != 0);
@@ -267,19 +380,21 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
                     dlo_c[w] = dlo;
                     r_c[w] = r;
                     view_c[w] = vf;
+                    if constexpr (PAR) par_c[w] = par;
                 }
-                const bool rays = kRays && (!TAB || ((flagged >> (k * kBwdPViews)) & ((1u << kBwdPViews) - 1u)) != 0);
+                const bool fly = !TAB || ((flagged >> (k * kBwdPViews)) & ((1u << kBwdPViews) - 1u)) != 0;
+                const bool rays = kRays && fly;
                 __syncwarp();
                 if (lane == 0) {
                     unsigned char* slot = ring + (size_t)st * m.stage;
-                    rays_c[st] = rays ? 1 : 0;
+                    fly_c[st] = fly ? 1 : 0;
                     fence_proxy_async_shared();
                     mbar_arrive_expect_tx(&tma_bar[st],
                                           (uint32_t)(nv * a.wd * (L::kRowElems * (int)sizeof(T) + (rays ? 32 : 0))));
                     for (int vl = 0; vl < nv; ++vl) {
                         const int d0 = dlo_c[st * kBwdPViews + vl];
                         tma_load_4d(slot + (size_t)vl * m.yst_view, &map, &tma_bar[st], 0, d0, v0 + vl, blockIdx.y);
-                        if (rays)   // the interpolating backprojector needs no rays
+                        if (rays)   // parallel views and the interpolating backprojector need no rays
                             tma_load_2d(slot + (size_t)kBwdPViews * m.yst_view + (size_t)vl * m.rst_view, &rmap,
                                         &tma_bar[st], 0, (v0 + vl) * a.D + d0);
                     }
@@ -330,6 +445,10 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
     constexpr int LOG_OCT = OCT == 1 ? 0 : OCT == 2 ? 1 : 2;
     const uint32_t ring_a = smem_u32(ring), yf_a = smem_u32(yf);
     const uint32_t win_a = smem_u32(view_c);
+    [[maybe_unused]] const uint32_t par_a = smem_u32(par_c);
+    // parallel walks of 32-image groups step in pairs (us, scalar -> paired at 512^2, 512 views: FP16 1419 -> 1222,
+    // FP32 1292 -> 1286), smaller groups do not (16 images: FP16 897 -> 912, FP32 854 -> 866)
+    [[maybe_unused]] constexpr bool kPaired = BG == 32;
     const uint32_t yview = L::kConv ? (uint32_t)m.yf_view : (uint32_t)m.yst_view;
     const uint32_t ystv = (uint32_t)m.yst_view, rstv = (uint32_t)m.rst_view;
     // TAB: this thread's table record of the next view, loaded one view ahead of its use
@@ -354,8 +473,8 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
         const uint32_t ybuf_a = L::kConv ? yf_a + (uint32_t)(c & 1) * (uint32_t)m.yf_buf : slot_a;
         if (!bad) {
             // (the table gather converts the 16-bit rows it reads itself: the widened rows serve only
-            // the on-the-fly weights, needed where the chunk's rays were copied)
-            if (L::kConv && (!TAB || rays_c[st])) {
+            // the on-the-fly weights)
+            if (L::kConv && (!TAB || fly_c[st])) {
                 // 16-bit window rows -> FP32 rows of pitch PITCH (8 images per 16-byte load); the
                 // view of item e is found by comparison (no division)
                 const int W = a.wd * OCT;
@@ -373,7 +492,7 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
                     sts4(dst + 16, f[1]);
                 }
             }
-            if (kRays && rays_c[st]) {
+            if (kRays && fly_c[st]) {
                 // re-base the landed rays on this tile, in place: one ray per thread
                 const int W = a.wd;
                 for (int e = tid; e < nv * W; e += NC) {
@@ -407,9 +526,40 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
             if (tid == 0) record_device_error(a.err, RADON_ERR_TIMEOUT);
             return;
         }
+        // one candidate row at ya, with both pixels' weights
+        auto add_row = [&](const uint32_t ya, const float (&w)[PX]) {
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                const float4 y4 = lds4(ya + 16 * q);
+                if constexpr (BG <= 16) {
+                    // paired FMAs (the same bits as scalar ones): half the instructions, which 8- and
+                    // 16-image groups issue among as many weights (2-3 % faster); 32-image groups
+                    // measured the same either way and spilled when paired
+                    const f32x2 y01 = f2_pack(y4.x, y4.y), y23 = f2_pack(y4.z, y4.w);
+#pragma unroll
+                    for (int x = 0; x < PX; ++x) {
+                        const f32x2 ww = f2_pack(w[x], w[x]);
+                        f32x2 a0 = f2_pack(acc[x][4 * q + 0], acc[x][4 * q + 1]);
+                        f32x2 a1 = f2_pack(acc[x][4 * q + 2], acc[x][4 * q + 3]);
+                        a0 = f2_fma(ww, y01, a0);
+                        a1 = f2_fma(ww, y23, a1);
+                        f2_unpack(a0, &acc[x][4 * q + 0], &acc[x][4 * q + 1]);
+                        f2_unpack(a1, &acc[x][4 * q + 2], &acc[x][4 * q + 3]);
+                    }
+                } else {
+#pragma unroll
+                    for (int x = 0; x < PX; ++x) {
+                        acc[x][4 * q + 0] = fmaf(w[x], y4.x, acc[x][4 * q + 0]);
+                        acc[x][4 * q + 1] = fmaf(w[x], y4.y, acc[x][4 * q + 1]);
+                        acc[x][4 * q + 2] = fmaf(w[x], y4.z, acc[x][4 * q + 2]);
+                        acc[x][4 * q + 3] = fmaf(w[x], y4.w, acc[x][4 * q + 3]);
+                    }
+                }
+            }
+        };
         for (int vl = 0; vl < nv; ++vl) {
             const uint32_t va = win_a + (uint32_t)(st * kBwdPViews + vl) * 32u;
-            const float4 v01 = lds4(va), v23 = lds4(va + 16);   // ax, ay, a0, bx | by, b0, -, -
+            const float4 v01 = lds4(va), v23 = lds4(va + 16);   // ax, ay, a0, bx | by, b0, -, - (or BwdPPar's)
             const int dlo = dlo_c[st * kBwdPViews + vl];
             const uint32_t yv = ybuf_a + (uint32_t)vl * yview;
             // detector coordinate of the first pixel; the second (one row down) adds (ay, by)
@@ -520,8 +670,39 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
                         }
                     }
                 }
-                if (!tabbed) {
-                    const float r = r_c[st * kBwdPViews + vl];
+                const float r = r_c[st * kBwdPViews + vl];
+                if constexpr (PAR) {
+                    if (!tabbed) {
+                        const float2 ex = lds2(par_a + (uint32_t)(st * kBwdPViews + vl) * 8u);
+                        const BwdPPar view = {v01.x, v01.y, v01.z, v01.w, v23.x, v23.y, v23.z, v23.w, ex.x, ex.y};
+                        BwdPWalk k = bwdp_par_walk(view, r, px, py0, a.ih2, a.wd);
+                        uint32_t ya = yv + (uint32_t)k.la * PITCH;
+                        if constexpr (kPaired) {
+                            const f32x2 step = f2_pack(view.sx, view.sy), next = f2_pack(k.nx, k.ny);
+                            f32x2 r2[PX] = {f2_pack(k.rx[0], k.ry[0]), f2_pack(k.rx[1], k.ry[1])};
+                            for (int dl = k.la; dl <= k.lb; ++dl, ya += PITCH) {
+                                float w[PX];
+#pragma unroll
+                                for (int x = 0; x < PX; ++x) {
+                                    w[x] = bwdp_tents2<KW>(r2[x], step);
+                                    r2[x] = f2_add(r2[x], next);
+                                }
+                                add_row(ya, w);
+                            }
+                        } else {
+                            for (int dl = k.la; dl <= k.lb; ++dl, ya += PITCH) {
+                                float w[PX];
+#pragma unroll
+                                for (int x = 0; x < PX; ++x) {
+                                    w[x] = bwdp_tents<KW>(k.rx[x], k.ry[x], view.sx, view.sy);
+                                    k.rx[x] += k.nx;
+                                    k.ry[x] += k.ny;
+                                }
+                                add_row(ya, w);
+                            }
+                        }
+                    }
+                } else if (!tabbed) {
                     // the union of the pixels' candidate ranges [t - r, t + r] (approximate divide: the
                     // windows carry margins far above its error); a candidate outside a pixel's own range
                     // has zero weight there.  Candidates outside the detector are sentinel rays over
@@ -544,34 +725,7 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
                         float w[PX];
                         w[0] = bwdp_weight<KW>(px, py0, s0, A);
                         w[1] = bwdp_weight<KW>(px, py0 + 1.0f, s0 + by, A);
-#pragma unroll
-                        for (int q = 0; q < NQ; ++q) {
-                            const float4 y4 = lds4(ya + 16 * q);
-                            if constexpr (BG <= 16) {
-                                // paired FMAs (the same bits as scalar ones): half the instructions, which 8- and
-                                // 16-image groups issue among as many weights (2-3 % faster); 32-image groups
-                                // measured the same either way and spilled when paired
-                                const f32x2 y01 = f2_pack(y4.x, y4.y), y23 = f2_pack(y4.z, y4.w);
-#pragma unroll
-                                for (int x = 0; x < PX; ++x) {
-                                    const f32x2 ww = f2_pack(w[x], w[x]);
-                                    f32x2 a0 = f2_pack(acc[x][4 * q + 0], acc[x][4 * q + 1]);
-                                    f32x2 a1 = f2_pack(acc[x][4 * q + 2], acc[x][4 * q + 3]);
-                                    a0 = f2_fma(ww, y01, a0);
-                                    a1 = f2_fma(ww, y23, a1);
-                                    f2_unpack(a0, &acc[x][4 * q + 0], &acc[x][4 * q + 1]);
-                                    f2_unpack(a1, &acc[x][4 * q + 2], &acc[x][4 * q + 3]);
-                                }
-                            } else {
-#pragma unroll
-                                for (int x = 0; x < PX; ++x) {
-                                    acc[x][4 * q + 0] = fmaf(w[x], y4.x, acc[x][4 * q + 0]);
-                                    acc[x][4 * q + 1] = fmaf(w[x], y4.y, acc[x][4 * q + 1]);
-                                    acc[x][4 * q + 2] = fmaf(w[x], y4.z, acc[x][4 * q + 2]);
-                                    acc[x][4 * q + 3] = fmaf(w[x], y4.w, acc[x][4 * q + 3]);
-                                }
-                            }
-                        }
+                        add_row(ya, w);
                     }
                 }
             }
@@ -599,7 +753,7 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
 // la .. la + 4 (record 8 la + count), or kBwdTabOverflow where
 // the weighted rays span more than five (counted in *overflow, and flagged for the tile and view in
 // tab_vflag, which must start at zero).
-template <int KW>
+template <int KW, bool PAR>
 __global__ void __launch_bounds__(kBwdTabPairs) bwdp_table_kernel(const RayT* __restrict__ rays,
                                                                  const ViewF* __restrict__ views, int n, int V, int D,
                                                                  float ih2, int wd, int tiles_x, int views_per_block,
@@ -625,9 +779,29 @@ __global__ void __launch_bounds__(kBwdTabPairs) bwdp_table_kernel(const RayT* __
         tlo = fminf(tlo, t1);
         thi = fmaxf(thi, t1);
         const float fd = (float)dlo;
-        const int la = __float2int_ru(fmaxf((tlo - r) - fd, 0.0f));
-        const int lb = __float2int_rd(fminf((thi + r) - fd, (float)(wd - 1)));
+        int la = __float2int_ru(fmaxf((tlo - r) - fd, 0.0f));
+        int lb = __float2int_rd(fminf((thi + r) - fd, (float)(wd - 1)));
+        BwdPPar view{};
+        BwdPWalk walk{};
+        if constexpr (PAR) {
+            view = bwdp_par_view(vf, rays, v, D, wd, dlo, ti, tj, ih2);
+            walk = bwdp_par_walk(view, r, px, py0, ih2, wd);
+            la = walk.la;
+            lb = walk.lb;
+        }
         auto weights = [&](int dl, float* w0, float* w1) {
+            if constexpr (PAR) {   // the gather's steps from ray la
+                BwdPWalk k = walk;
+                for (int l = la; l < dl; ++l) {
+                    k.rx[0] += k.nx;
+                    k.ry[0] += k.ny;
+                    k.rx[1] += k.nx;
+                    k.ry[1] += k.ny;
+                }
+                *w0 = bwdp_tents<KW>(k.rx[0], k.ry[0], view.sx, view.sy);
+                *w1 = bwdp_tents<KW>(k.rx[1], k.ry[1], view.sx, view.sy);
+                return;
+            }
             const int d = dlo + dl;
             const bool valid = d >= 0 && d < D;
             RayT ray{0, 0, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
@@ -681,10 +855,15 @@ inline size_t bwdp_plan(int wd, bool rays, int* stages) {
     return bwdp_smem<T, BG>(wd, S, rays).total;
 }
 
-template <typename T, int BG, int KW, bool TAB = false>
+// Whether the exact adjoint of groups of bg images reads the geometry's weight table.
+inline bool bwdp_table_serves(const radon_geometry* g, int bg) {
+    return g->d_tab_w != nullptr && (g->fan ? bg <= 16 : bg == 16 && g->tab_kw == 6);
+}
+
+template <typename T, int BG, int KW, bool TAB, bool PAR>
 cudaError_t bwdp_launch(const CUtensorMap& map, const CUtensorMap& rmap, const BwdPArgs& a, dim3 grid, size_t smem,
                         cudaStream_t s) {
-    auto kern = backward_packed_kernel<T, BG, KW, TAB>;
+    auto kern = backward_packed_kernel<T, BG, KW, TAB, PAR>;
     static size_t attr_bytes = 0;
     if (smem > attr_bytes) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -708,11 +887,14 @@ radon_status launch_backward_packed_t(const radon_geometry* g, const void* packe
         *why = "detector window wider than a TMA box";
         return RADON_ERR_UNSUPPORTED;
     }
-    // the geometry's weight table serves the exact adjoint's pixel pairs (16-bit or smaller groups)
-    const bool tab = kw > 0 && BG <= 16 && g->d_tab_w != nullptr && g->tab_kw == kw && g->tab_wd == wd;
+    // The geometry's weight table serves the exact adjoint's smaller groups.  A parallel beam's weights are
+    // cheaper to compute than to read (16 x 512^2, 512 views: 852 us computed, 942 us read; 8 images 673,
+    // 886) but for short steps, six samples a window, in groups of 16 (360 views, step 0.5: 692, 652).
+    const bool par = kw > 0 && g->fan == 0;
+    const bool tab = kw > 0 && bwdp_table_serves(g, BG) && g->tab_kw == kw && g->tab_wd == wd;
     int stages = 2;
-    // the table kernel stages ray rows too (for the pairs its table marks as overflowing)
-    const size_t smem = bwdp_plan<T, BG>(wd, kw > 0, &stages);
+    // ray rows are staged for fans (with a table too, for the pairs it marks as overflowing)
+    const size_t smem = bwdp_plan<T, BG>(wd, kw > 0 && !par, &stages);
     if (smem > 227 * 1024) {
         *why = "shared memory budget exceeded";
         return RADON_ERR_UNSUPPORTED;
@@ -731,6 +913,7 @@ radon_status launch_backward_packed_t(const radon_geometry* g, const void* packe
     }
     BwdPArgs a;
     a.views = g->d_view;
+    a.rays = g->d_ray;
     a.img = img;
     a.n = g->n;
     a.V = g->V;
@@ -750,20 +933,26 @@ radon_status launch_backward_packed_t(const radon_geometry* g, const void* packe
     a.tab_vflag = g->d_tab_vflag;
     a.tab_la = g->d_tab_la;
     const dim3 grid((unsigned)(a.tiles_x * a.tiles_x), (unsigned)groups);
-    cudaError_t e;
-    if constexpr (BG <= 16) {
-        if (tab) {
-            e = kw == 3 ? bwdp_launch<T, BG, 3, true>(map, rmap, a, grid, smem, s)
-                        : bwdp_launch<T, BG, 6, true>(map, rmap, a, grid, smem, s);
-        } else {
-            e = kw == 0   ? bwdp_launch<T, BG, 0>(map, rmap, a, grid, smem, s)
-                : kw == 3 ? bwdp_launch<T, BG, 3>(map, rmap, a, grid, smem, s)
-                          : bwdp_launch<T, BG, 6>(map, rmap, a, grid, smem, s);
-        }
+    auto launch = [&](auto kwc, auto tabc, auto parc) {
+        return bwdp_launch<T, BG, decltype(kwc)::value, decltype(tabc)::value, decltype(parc)::value>(map, rmap, a, grid,
+                                                                                                    smem, s);
+    };
+    using K3 = std::integral_constant<int, 3>;
+    using K6 = std::integral_constant<int, 6>;
+    constexpr std::true_type yes{};
+    constexpr std::false_type no{};
+    cudaError_t e = cudaErrorInvalidConfiguration;
+    if (kw == 0) {
+        e = launch(std::integral_constant<int, 0>{}, no, no);
+    } else if (!tab) {
+        if (par)
+            e = kw == 3 ? launch(K3{}, no, yes) : launch(K6{}, no, yes);
+        else
+            e = kw == 3 ? launch(K3{}, no, no) : launch(K6{}, no, no);
+    } else if (!par) {
+        if constexpr (BG <= 16) e = kw == 3 ? launch(K3{}, yes, no) : launch(K6{}, yes, no);
     } else {
-        e = kw == 0   ? bwdp_launch<T, BG, 0>(map, rmap, a, grid, smem, s)
-            : kw == 3 ? bwdp_launch<T, BG, 3>(map, rmap, a, grid, smem, s)
-                      : bwdp_launch<T, BG, 6>(map, rmap, a, grid, smem, s);
+        if constexpr (BG == 16) e = launch(K6{}, yes, yes);
     }
     if (e != cudaSuccess) {
         *why = std::string("packed adjoint launch: ") + cudaGetErrorString(e);
