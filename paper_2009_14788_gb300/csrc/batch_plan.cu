@@ -42,7 +42,8 @@ namespace {
 
 constexpr uint64_t kPlanMagic = 0x5241444f4e504c4eULL;   // "RADONPLN"
 constexpr int kPlanThreads = 256;
-constexpr int kAdjThreads = 128;     // adjoint: each thread owns a vertical pair of a 16 x 16 tile's pixels
+// Adjoint: threads of a CTA that own px (2: a vertical pair, 1) of a 16 x 16 tile's pixels each.
+constexpr int adj_threads(int px) { return kBwdTile * kBwdTile / px; }
 constexpr int kMaxChunkViews = 32;   // adjoint: views per staged chunk at most (16 where 32 do not fit)
 
 struct Unit {
@@ -269,14 +270,22 @@ __device__ __forceinline__ void plan_forward_tile(const Unit& u, int tile, const
     }
 }
 
+// Next work item of a persistent CTA: its own index first, then the counter's.  CTAs start spread over the SMs,
+// so the longest items (the list's first) do too, and a launch of no more CTAs than items leaves none idle
+// beside a full one: taken from the counter alone, the first items went to the first SMs' CTAs (adjoint of
+// 371^2 with 675 views and 106^2 with 230, 625 items: 475 -> 314 us with a pair of pixels per thread).
+__device__ __forceinline__ int next_work(bool first, unsigned* counter) {
+    return first ? (int)blockIdx.x : (int)(gridDim.x + atomicAdd(counter, 1u));
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kPlanThreads, 6) plan_forward_kernel(const Unit* __restrict__ units,
                                                                     const Work* __restrict__ work, int n_work,
                                                                     unsigned* counter,
                                                                     const typename Quad<T>::type* __restrict__ quads) {
     __shared__ int s_w;
-    for (;;) {
-        if (threadIdx.x == 0) s_w = (int)atomicAdd(counter, 1u);
+    for (bool first = true;; first = false) {
+        if (threadIdx.x == 0) s_w = next_work(first, counter);
         __syncthreads();
         const int wi = s_w;
         __syncthreads();
@@ -340,30 +349,36 @@ __device__ __forceinline__ AdjBuffers adj_buffers(unsigned char* smem_raw, int m
     return b;
 }
 
-// Tile-local pixels of thread `tid`: (pi, pj) and the one below it.  Each warp takes an 8 x 8 block, each
-// group of eight lanes (one 16-byte shared-load phase) a 4 x 4 block.
-__device__ __forceinline__ void adj_pair_of(int tid, int* pi, int* pj) {
+// Tile-local pixels of thread `tid`.  Two pixels: (pi, pj) and the one below it, each warp an 8 x 8 block, each
+// group of eight lanes (one 16-byte shared-load phase) a 4 x 4 block.  One: warps of 4 x 8, groups of 4 x 2.
+template <int PX>
+__device__ __forceinline__ void adj_pixels_of(int tid, int* pi, int* pj) {
     const int warp = tid >> 5, lane = tid & 31;
     const int grp = lane >> 3, e8 = lane & 7;
+    if constexpr (PX == 1) {
+        *pi = (warp >> 1) * 4 + (e8 >> 1);
+        *pj = (warp & 1) * 8 + grp * 2 + (e8 & 1);
+        return;
+    }
     *pi = (warp >> 1) * 8 + ((grp >> 1) * 2 + (e8 >> 2)) * 2;
     *pj = (warp & 1) * 8 + (grp & 1) * 4 + (e8 & 3);
 }
 
 // Work item `tile` of unit u (a 16 x 16 pixel tile over all views), stored through the epilogue
 // (the identity for plans).  Every thread of the CTA calls it (it holds CTA barriers).  Fan beams.
-template <typename T, int KW>
+template <typename T, int KW, int PX>
 __device__ void plan_adjoint_tile(const Unit& u, int tile, const AdjBuffers& b, const Epilogue& ep, int* err) {
     const int tid = threadIdx.x;
     int pi0, pj;
-    adj_pair_of(tid, &pi0, &pj);
+    adj_pixels_of<PX>(tid, &pi0, &pj);
     const int tiles_x = (u.n + kBwdTile - 1) / kBwdTile;
     const int ti = (tile / tiles_x) * kBwdTile, tj = (tile - (tile / tiles_x) * tiles_x) * kBwdTile;
     const float gx = (float)(tj + pj);
     const f32x2 ih2_2 = f2_pack(u.ih2, u.ih2);
     const T* y = static_cast<const T*>(u.in);
     const int CV = u.cfg, wd = u.wd;
-    float acc[2] = {0.0f, 0.0f};
-    bool viol[2] = {false, false};
+    float acc[PX] = {};
+    bool viol[PX] = {};
     for (int c0 = 0; c0 < u.V; c0 += CV) {
         const int nv = min(CV, u.V - c0);
         if (tid < nv) {
@@ -376,7 +391,7 @@ __device__ void plan_adjoint_tile(const Unit& u, int tile, const AdjBuffers& b, 
             b.sh->r[tid] = r;
         }
         __syncthreads();
-        for (int e = tid; e < nv * wd; e += kAdjThreads) {
+        for (int e = tid; e < nv * wd; e += adj_threads(PX)) {
             const int vl = e / wd, dl = e - (e / wd) * wd;
             const int d = b.sh->dlo[vl] + dl;
             const bool valid = d >= 0 && d < u.D;
@@ -396,7 +411,7 @@ __device__ void plan_adjoint_tile(const Unit& u, int tile, const AdjBuffers& b, 
             const float* yv = b.ys + vl * wd;
             const float* cv = b.rc + vl * wd;
 #pragma unroll
-            for (int x = 0; x < 2; ++x) {
+            for (int x = 0; x < PX; ++x) {
                 const float px = (float)pj, py = (float)(pi0 + x), gy = (float)(ti + pi0 + x);
                 const f32x2 p2 = f2_pack(px, py);
                 const float num = fmaf(vf.ax, gx, fmaf(vf.ay, gy, vf.a0));
@@ -415,7 +430,7 @@ __device__ void plan_adjoint_tile(const Unit& u, int tile, const AdjBuffers& b, 
         __syncthreads();
     }
 #pragma unroll
-    for (int x = 0; x < 2; ++x) {
+    for (int x = 0; x < PX; ++x) {
         if ((ti + pi0 + x) >= u.n || (tj + pj) >= u.n) continue;
         if (viol[x]) record_device_error(err, RADON_ERR_DEVICE_BOUNDS);
         const long long idx = (long long)(ti + pi0 + x) * u.n + (tj + pj);
@@ -439,19 +454,22 @@ __device__ void plan_adjoint_tile(const Unit& u, int tile, const AdjBuffers& b, 
 // both, the second pixel's coordinates are one addition away, the nearest-integer of a coordinate shifted
 // by 1/2 (adding and subtracting 1.5 * 2^23) takes the place of the conversions and clamps, and
 // eight CTAs of 128 threads hold a whole 512^2 image in one wave.
-template <typename T, int KW, int NC>
+// PX = 1: one pixel per thread, the same bits: the lower pixel of a pair still adds to the upper's coordinates.
+template <typename T, int KW, int NC, int PX>
 __device__ void plan_adjoint_tile_parallel(const Unit& u, int tile, const AdjBuffers& b, const Epilogue& ep,
                                            int* err) {
     constexpr float kMagic = 12582912.0f;        // 1.5 * 2^23: x + kMagic rounds x to the nearest integer
     constexpr unsigned kMagicBits = 0x4B400000u;
     const int tid = threadIdx.x;
     int pi0, pj;
-    adj_pair_of(tid, &pi0, &pj);
+    adj_pixels_of<PX>(tid, &pi0, &pj);
     const int tiles_x = (u.n + kBwdTile - 1) / kBwdTile;
     const int ti = (tile / tiles_x) * kBwdTile, tj = (tile - (tile / tiles_x) * tiles_x) * kBwdTile;
     // pixels past the image's edge repeat the edge's: every coordinate stays within the tile's corners
     const int xe = min(kBwdTile - 1, u.n - 1 - tj), ye = min(kBwdTile - 1, u.n - 1 - ti);
-    const float px = (float)min(pj, xe), py0 = (float)min(pi0, ye), py1 = (float)min(pi0 + 1, ye);
+    const int pe = PX == 2 ? pi0 : pi0 & ~1;     // the pair's upper row
+    const float px = (float)min(pj, xe), py0 = (float)min(pe, ye);
+    const float py1 = PX == 1 && pe == pi0 ? py0 : (float)min(pe + 1, ye);
     const f32x2 np0 = f2_pack(-px, -py0), np1 = f2_pack(-px, -py1);
     const float dy = py1 - py0;
     const T* y = static_cast<const T*>(u.in);
@@ -508,7 +526,7 @@ __device__ void plan_adjoint_tile_parallel(const Unit& u, int tile, const AdjBuf
             b.sh->r[tid] = r;
         }
         __syncthreads();
-        for (int e = tid; e < nv * wp; e += kAdjThreads) {
+        for (int e = tid; e < nv * wp; e += adj_threads(PX)) {
             int vl = (int)((float)e * inv_wp);   // e / wp, corrected for the quotient's rounding
             vl -= vl * wp > e;
             vl += (vl + 1) * wp <= e;
@@ -544,13 +562,16 @@ __device__ void plan_adjoint_tile_parallel(const Unit& u, int tile, const AdjBuf
             };
             if constexpr (NC > 0) {
                 const float m0 = t0 + kMagic, m1 = t1 + kMagic;
-                f32x2 ra = first(np0, ka0, m0 - kMagic), rb = first(np1, ka1, m1 - kMagic);
+                [[maybe_unused]] f32x2 ra = first(np0, ka0, m0 - kMagic);
+                f32x2 rb = first(np1, ka1, m1 - kMagic);
                 const uint32_t ya = yb + 4u * __float_as_uint(m0), yc = yb + 4u * __float_as_uint(m1);
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
-                    acc0 = fmaf(weight(ra), lds1(ya + 4u * c), acc0);
+                    if constexpr (PX == 2) {
+                        acc0 = fmaf(weight(ra), lds1(ya + 4u * c), acc0);
+                        ra = f2_add(ra, dn2);
+                    }
                     acc1 = fmaf(weight(rb), lds1(yc + 4u * c), acc1);
-                    ra = f2_add(ra, dn2);
                     rb = f2_add(rb, dn2);
                 }
             } else {
@@ -566,58 +587,67 @@ __device__ void plan_adjoint_tile_parallel(const Unit& u, int tile, const AdjBuf
                         r2 = f2_add(r2, dn2);
                     }
                 };
-                loop(np0, t0, ka0, acc0);
+                if constexpr (PX == 2) loop(np0, t0, ka0, acc0);
                 loop(np1, t1, ka1, acc1);
             }
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int x = 0; x < 2; ++x) {
+    for (int x = 0; x < PX; ++x) {
         if ((ti + pi0 + x) >= u.n || (tj + pj) >= u.n) continue;
         const long long idx = (long long)(ti + pi0 + x) * u.n + (tj + pj);
-        static_cast<T*>(u.out)[idx] = from_f32<T>(epilogue_value<T>(ep, u.h * (x ? acc1 : acc0), idx));
+        static_cast<T*>(u.out)[idx] = from_f32<T>(epilogue_value<T>(ep, u.h * (x == PX - 1 ? acc1 : acc0), idx));
     }
 }
 
-// Eight CTAs of 128 threads per SM: the launch bounds keep both geometry kinds within 64 registers.
-template <typename T, int KW>
-__global__ void __launch_bounds__(kAdjThreads, 8) plan_adjoint_kernel(const Unit* __restrict__ units,
+// 1024 threads per SM: the launch bounds keep both geometry kinds within 64 registers.
+template <typename T, int KW, int PX>
+__global__ void __launch_bounds__(adj_threads(PX), 4 * PX) plan_adjoint_kernel(const Unit* __restrict__ units,
                                                                     const Work* __restrict__ work, int n_work,
                                                                     unsigned* counter, int max_wd, int cap, int* err) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const AdjBuffers b = adj_buffers(smem_raw, max_wd, cap);
-    for (;;) {
+    for (bool first = true;; first = false) {
         // the previous tile's last barrier orders its reads of `w` before this write
-        if (threadIdx.x == 0) b.sh->w = (int)atomicAdd(counter, 1u);
+        if (threadIdx.x == 0) b.sh->w = next_work(first, counter);
         __syncthreads();
         const int wi = b.sh->w;
         if (wi >= n_work) return;
         const Work w = work[wi];
         const Unit& u = units[w.unit];
         if (u.fan)
-            plan_adjoint_tile<T, KW>(u, w.tile, b, Epilogue{1.0f, nullptr, 0.0f, nullptr}, err);
+            plan_adjoint_tile<T, KW, PX>(u, w.tile, b, Epilogue{1.0f, nullptr, 0.0f, nullptr}, err);
         else if (u.cand3)
-            plan_adjoint_tile_parallel<T, KW, 3>(u, w.tile, b, Epilogue{1.0f, nullptr, 0.0f, nullptr}, err);
+            plan_adjoint_tile_parallel<T, KW, 3, PX>(u, w.tile, b, Epilogue{1.0f, nullptr, 0.0f, nullptr}, err);
         else
-            plan_adjoint_tile_parallel<T, KW, 0>(u, w.tile, b, Epilogue{1.0f, nullptr, 0.0f, nullptr}, err);
+            plan_adjoint_tile_parallel<T, KW, 0, PX>(u, w.tile, b, Epilogue{1.0f, nullptr, 0.0f, nullptr}, err);
     }
 }
 
 // Single image (a batch-1 call): one CTA per tile, the unit passed by value.  NC < 0: fan beam.
-template <typename T, int KW, int NC>
-__global__ void __launch_bounds__(kAdjThreads, 8) single_adjoint_kernel(const Unit u, const Epilogue ep, int* err) {
+template <typename T, int KW, int NC, int PX>
+__global__ void __launch_bounds__(adj_threads(PX), 4 * PX) single_adjoint_kernel(const Unit u, const Epilogue ep, int* err) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if constexpr (NC < 0)
-        plan_adjoint_tile<T, KW>(u, (int)blockIdx.x, adj_buffers(smem_raw, u.wd, u.cfg), ep, err);
+        plan_adjoint_tile<T, KW, PX>(u, (int)blockIdx.x, adj_buffers(smem_raw, u.wd, u.cfg), ep, err);
     else
-        plan_adjoint_tile_parallel<T, KW, NC>(u, (int)blockIdx.x, adj_buffers(smem_raw, u.wd, u.cfg), ep, err);
+        plan_adjoint_tile_parallel<T, KW, NC, PX>(u, (int)blockIdx.x, adj_buffers(smem_raw, u.wd, u.cfg), ep, err);
 }
 
 size_t adj_smem_bytes(int max_wd, int cap) {
     // parallel-beam units use the window constants' space past their values for the kAdjPad zeros
     return (sizeof(AdjShared) + 15) / 16 * 16 + (size_t)cap * max_wd * (16 + 4 + 4);
 }
+
+constexpr int kAdjSms = 152;
+
+// Pixels per thread of a parallel-beam adjoint launch with the work of `tiles` tiles as long as its longest: a
+// pair is less work, single pixels twice the warps, which a launch of few tiles wants (us, single -> pair:
+// one image of 64^2 36 -> 42, 256^2 48 -> 48, 448^2, 5.2 tiles per SM, 120 -> 115, 512^2 138 -> 132; plans
+// of 0.7 tiles per SM 98 -> 121, 3.9 289 -> 314, 4.5 186 -> 173, 8.9 471 -> 456, 12.7 260 -> 229).  Fans' pairs
+// share little and are never the faster (64^2 112 -> 176, 576^2 494 -> 515).
+int adj_pixels(double tiles, int sms) { return tiles >= 4.5 * sms ? 2 : 1; }
 
 // Views per chunk at most for windows of max_wd rays: 32 where the staging fits one CTA's shared
 // memory, else 16; 0 if not even 16 fit.
@@ -802,17 +832,24 @@ radon_status single_forward_t(const radon_geometry* g, const void* img, void* si
     return RADON_OK;
 }
 
-template <typename T, int KW, int NC>
-radon_status single_backward_tk(const Unit& u, long long tiles, size_t smem, const Epilogue& ep, int* err,
+template <typename T, int KW, int NC, int PX>
+radon_status single_backward_px(const Unit& u, long long tiles, size_t smem, const Epilogue& ep, int* err,
                                 cudaStream_t s) {
-    auto kern = single_adjoint_kernel<T, KW, NC>;
-    const cudaError_t ea = raise_smem_attr<single_adjoint_kernel<T, KW, NC>>(smem);
+    auto kern = single_adjoint_kernel<T, KW, NC, PX>;
+    const cudaError_t ea = raise_smem_attr<single_adjoint_kernel<T, KW, NC, PX>>(smem);
     if (ea != cudaSuccess) return cuda_fail(ea, "single-image adjoint shared memory");
-    kern<<<(unsigned)tiles, kAdjThreads, smem, s>>>(u, ep, err);
+    kern<<<(unsigned)tiles, adj_threads(PX), smem, s>>>(u, ep, err);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "single-image adjoint launch");
     count_launches(1);
     return RADON_OK;
+}
+
+template <typename T, int KW, int NC>
+radon_status single_backward_tk(const Unit& u, long long tiles, size_t smem, const Epilogue& ep, int* err,
+                                cudaStream_t s) {
+    return NC >= 0 && adj_pixels((double)tiles, kAdjSms) == 2 ? single_backward_px<T, KW, NC, 2>(u, tiles, smem, ep, err, s)
+                                                   : single_backward_px<T, KW, NC, 1>(u, tiles, smem, ep, err, s);
 }
 
 template <typename T>
@@ -881,6 +918,7 @@ struct radon_plan {
     radon_dtype dtype = RADON_F32;
     int device = 0;
     int kw = 3;
+    int px = 2;                 // adjoint: pixels per thread
     int max_wd = 0;
     int cap = kMaxChunkViews;   // adjoint: views per chunk at most (its shared memory holds that many)
     int ctas = 0;
@@ -995,7 +1033,7 @@ radon_status launch_t(const radon_plan* p, const Work* d_work, int n_work, int n
             count_launches(1);
         }
         if (n_work > n_staged)
-            plan_forward_kernel<T><<<p->ctas, kPlanThreads, 0, s>>>(p->d_units, d_work + n_staged, n_work - n_staged,
+            plan_forward_kernel<T><<<std::min(p->ctas, n_work - n_staged), kPlanThreads, 0, s>>>(p->d_units, d_work + n_staged, n_work - n_staged,
                                                                    p->d_counter + 1, static_cast<const Q*>(p->d_quads));
         e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "plan forward launch");
@@ -1003,12 +1041,10 @@ radon_status launch_t(const radon_plan* p, const Work* d_work, int n_work, int n
     } else {
         int* err = device_error_word();
         if (err == nullptr) return fail(RADON_ERR_CUDA, "device error word unavailable");
-        if (p->kw == 3)
-            plan_adjoint_kernel<T, 3><<<p->ctas, kAdjThreads, p->smem, s>>>(p->d_units, d_work, n_work, p->d_counter,
-                                                                            p->max_wd, p->cap, err);
-        else
-            plan_adjoint_kernel<T, 6><<<p->ctas, kAdjThreads, p->smem, s>>>(p->d_units, d_work, n_work, p->d_counter,
-                                                                            p->max_wd, p->cap, err);
+        auto kern = p->px == 2 ? (p->kw == 3 ? plan_adjoint_kernel<T, 3, 2> : plan_adjoint_kernel<T, 6, 2>)
+                               : (p->kw == 3 ? plan_adjoint_kernel<T, 3, 1> : plan_adjoint_kernel<T, 6, 1>);
+        kern<<<std::min(p->ctas, n_work), adj_threads(p->px), p->smem, s>>>(p->d_units, d_work, n_work, p->d_counter, p->max_wd, p->cap,
+                                                         err);
         e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "plan adjoint launch");
         count_launches(1);
@@ -1022,6 +1058,13 @@ radon_status launch_plan(const radon_plan* p, const Work* d_work, int n_work, in
         case RADON_BF16: return launch_t<__nv_bfloat16>(p, d_work, n_work, n_staged, s);
         default: return launch_t<float>(p, d_work, n_work, n_staged, s);
     }
+}
+
+template <typename T, int KW, int PX>
+cudaError_t adj_occupancy(size_t smem, int* per_sm) {
+    const cudaError_t e = raise_smem_attr<plan_adjoint_kernel<T, KW, PX>>(smem);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, plan_adjoint_kernel<T, KW, PX>, adj_threads(PX), smem);
 }
 
 template <typename T>
@@ -1041,14 +1084,18 @@ radon_status occupancy_t(radon_plan* p) {
     }
     if (p->direction == 0) {
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, plan_forward_kernel<T>, kPlanThreads, 0);
-    } else if (p->kw == 3) {
-        e = raise_smem_attr<plan_adjoint_kernel<T, 3>>(p->smem);
-        if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, plan_adjoint_kernel<T, 3>, kAdjThreads, p->smem);
     } else {
-        e = raise_smem_attr<plan_adjoint_kernel<T, 6>>(p->smem);
-        if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, plan_adjoint_kernel<T, 6>, kAdjThreads, p->smem);
+        // the whole work in tiles of the longest unit's views
+        double all = 0.0, fan = 0.0, longest = 1.0;
+        for (const Unit& u : p->units) {
+            const int t = (u.n + kBwdTile - 1) / kBwdTile;
+            all += (double)t * t * u.V;
+            if (u.fan) fan += (double)t * t * u.V;
+            longest = std::max(longest, (double)u.V);
+        }
+        p->px = 2 * fan > all ? 1 : adj_pixels(all / longest, sms);
+        e = p->px == 2 ? (p->kw == 3 ? adj_occupancy<T, 3, 2>(p->smem, &per_sm) : adj_occupancy<T, 6, 2>(p->smem, &per_sm))
+                       : (p->kw == 3 ? adj_occupancy<T, 3, 1>(p->smem, &per_sm) : adj_occupancy<T, 6, 1>(p->smem, &per_sm));
     }
     if (e != cudaSuccess) return cuda_fail(e, "plan occupancy query");
     p->ctas = std::max(1, per_sm) * sms;
