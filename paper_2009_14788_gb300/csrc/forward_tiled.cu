@@ -9,6 +9,7 @@ namespace radon {
 namespace {
 
 constexpr uint32_t kSpinLimit = 1u << 22;   // bounded mbarrier polls (~seconds) before giving up
+constexpr long long kFwdFourMinCtas = 300;   // CTAs of four texel groups below which smaller ones fill the GPU better
 
 // FP16 storage takes FP16 weights in mixed-precision FMAs only when the config asks for them and the
 // epilogue adds nothing to the projection (a fused residual keeps FP32 weights); the default is FP32.
@@ -206,12 +207,26 @@ radon_status packed_forward_shape(radon_geometry* g, radon_dtype dt, int batch, 
     // about what a pair and a single do) and FP32 batches of more than 16 (2.33 -> 1.56 ms; 32 x 256^2, 256
     // views 376 -> 242 us; smaller FP32 batches keep the one group that the query reports for them), in
     // the highest slab of 8, 6 or 4 rows that leaves two CTAs per SM (8 rows 1.45 ms, 6 1.48, 4 1.56; 10
-    // rows at one CTA 1.88).  FP16 weights keep two groups.
+    // rows at one CTA 1.88).  FP16 weights keep two groups.  Not where the CTAs of four groups would not fill
+    // two per SM (us, default -> four groups, FP16: 32 x 256^2, 128 views, 204 CTAs 177 -> 194; 192 views, 300
+    // CTAs 242 -> 239; 256 views, 396 CTAs 284 -> 246), nor, since a CTA costs the same with empty groups and
+    // thin slabs repeat the rows between them, where groups are empty and the slab is low: FP32, against one
+    // group per CTA, needs 6 rows (32 x 512^2, 100 views, 4 rows: 682 -> 891; 32 x 256^2, 128 views, 6 rows:
+    // 219 -> 178), either type two more with two groups empty (FP32 24 x 256^2, 256 views, 8 rows: 289 -> 239;
+    // 24 x 266^2 fan, 586 views, 6 rows: 570 -> 640) and FP32 never runs with three (20 x 512^2, 150 views:
+    // 579 -> 958).
+    const int groups = (batch + BG - 1) / BG;
+    const int empty = groups < 12 ? (4 - groups % 4) % 4 : 0;   // (of many, a few cost little)
+    const int min_rows = 4 + (esz == 4 ? 2 : 0) + (empty >= 2 ? 2 : 0);
+    const long long ctas4 = (long long)g->group_count[G >= 8 ? 3 : G >= 4 ? 2 : G >= 2 ? 1 : 0] * ((g->D + Dt - 1) / Dt) *
+                            ((groups + 3) / 4);
+    const int fixed_rows = cfg ? cfg->rows_per_slab : 0;
+    const bool four = !f16w && batch > (esz == 2 ? 24 : 16) && !(esz == 4 && empty == 3) && ctas4 >= kFwdFourMinCtas &&
+                      (fixed_rows == 0 || fixed_rows >= min_rows);
     int NG = lanes == 2 ? 1
              : ipc != 0 ? (ipc == 2 * BG ? 2 : 1)
-             : !f16w && batch > (esz == 2 ? 24 : 16) ? 4
-                                                     : (esz == 2 && batch > BG ? 2 : 1);
-    const int fixed_rows = cfg ? cfg->rows_per_slab : 0;
+             : four     ? 4
+                        : (esz == 2 && batch > BG ? 2 : 1);
     int R = fixed_rows ? fixed_rows : 8;   // of four groups, lowered until they fit
     for (;;) {
         if (NG != 4) R = fixed_rows ? fixed_rows : (NG == 2 ? (f16w ? 8 : 14) : 16);
@@ -228,7 +243,7 @@ radon_status packed_forward_shape(radon_geometry* g, radon_dtype dt, int batch, 
         while (stages < kFwdMaxStages && fwd_packed_smem_bytes(R, wbox, stages + 1, NG) <= room) ++stages;
         const size_t smem = fwd_packed_smem_bytes(R, wbox, stages, NG);
         if (NG == 4 && (wbox > 256 || smem > room)) {
-            if (!fixed_rows && R > 4) R -= 2;
+            if (!fixed_rows && R > min_rows) R -= 2;
             else NG = esz == 2 ? 2 : 1;
             continue;
         }
