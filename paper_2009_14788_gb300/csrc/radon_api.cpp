@@ -199,24 +199,24 @@ radon_status validate_epilogue(const radon_epilogue* e, radon_dtype dt) {
 
 }  // namespace
 
-// The packed forward's config with `views` views per CTA; images per CTA: one texel group or two (a value
-// meant for the adjoint leaves the default).
-radon_launch_config packed_forward_config(const radon_launch_config* cfg, radon_dtype dt, int views) {
+// The packed forward's config for one try; images per CTA: the caller's one texel group or two (a value
+// meant for the adjoint leaves the default), else the try's.
+radon_launch_config packed_forward_config(const radon_launch_config* cfg, radon_dtype dt, const PackedTry& t) {
     const int bg = dt == RADON_F32 ? 4 : 8;
     const int ipc = cfg != nullptr && (cfg->images_per_cta == bg || cfg->images_per_cta == 2 * bg)
-                        ? cfg->images_per_cta : 0;
-    return radon_launch_config{RADON_ALGO_TILED, views, cfg ? cfg->rows_per_slab : 0, ipc, 0, 0, cfg ? cfg->weights : 0};
+                        ? cfg->images_per_cta : t.images;
+    return radon_launch_config{RADON_ALGO_TILED, t.views, cfg ? cfg->rows_per_slab : 0, ipc, 0, 0, cfg ? cfg->weights : 0};
 }
 
 int packed_forward_tries(radon_geometry* g, radon_dtype dt, int batch, const radon_launch_config* cfg, bool f16w,
                          PackedTry* out) {
     if (cfg != nullptr && cfg->views_per_cta != 0) {
-        out[0] = PackedTry{cfg->views_per_cta, 1};
+        out[0] = PackedTry{cfg->views_per_cta, 1, 0};
         return 1;
     }
     int n = 0;
     const int bg = dt == RADON_F32 ? 4 : 8;
-    const radon_launch_config c8 = packed_forward_config(cfg, dt, 8);
+    const radon_launch_config c8 = packed_forward_config(cfg, dt, PackedTry{8, 1, 0});
     PackedFwdShape sh;
     std::string why;
     if (batch <= bg && c8.images_per_cta != 2 * bg &&
@@ -226,10 +226,21 @@ int packed_forward_tries(radon_geometry* g, radon_dtype dt, int batch, const rad
         // CTAs of 120 views: 178 against 183).  FP32 bands take twice the copies per image: only where
         // not even one CTA per SM runs (4 x 128^2, 128 views, 96 CTAs: 33 -> 28 us; 184 CTAs: 157 against 174).
         const long long ctas = (long long)g->group_count[3] * ((g->D + sh.Dt - 1) / sh.Dt);
-        if (ctas < (dt == RADON_F32 ? 152 : 2 * 152)) out[n++] = PackedTry{4, 2};
+        if (ctas < (dt == RADON_F32 ? 152 : 2 * 152)) out[n++] = PackedTry{4, 2, 0};
+    }
+    if (batch > bg && !f16w && c8.images_per_cta == 0 && c8.rows_per_slab == 0 &&
+        packed_forward_shape(g, dt, batch, &c8, false, 1, &sh, &why) == RADON_OK && sh.NG == 2) {
+        // A pair of texel groups shares each sample's index work, but where its bands leave an SM one CTA, or
+        // its CTAs are fewer than the SMs, twice the CTAs of one group are faster (us, pair -> single, 16 FP16
+        // images: 512^2, 150 views, 1 CTA per SM 426 -> 384; 360-view fan 883 -> 842; 384^2, 128 views 230 ->
+        // 197; 128^2, 128 views, 108 CTAs 59 -> 54; two CTAs per SM: 512^2, 512 views 962 -> 1056; 24 BF16
+        // images: 512^2, 150 views 568 -> 488, but on few CTAs, 256^2, 64 views, 104 -> 120).
+        const long long ctas = (long long)g->group_count[3] * ((g->D + sh.Dt - 1) / sh.Dt) * ((batch + 2 * bg - 1) / (2 * bg));
+        const bool wide = 2 * (sh.smem + 1024) > 228 * 1024 && (ctas >= 2 * 152 || batch <= 2 * bg);
+        if (wide || ctas < 152) out[n++] = PackedTry{8, 1, bg};
     }
     for (int lanes = 1; lanes <= 2; ++lanes)
-        for (int views = 8; views >= 1; views /= 2) out[n++] = PackedTry{views, lanes};
+        for (int views = 8; views >= 1; views /= 2) out[n++] = PackedTry{views, lanes, 0};
     return n;
 }
 
@@ -315,7 +326,7 @@ radon_status project(const radon_geometry* g, const void* in, void* out, radon_d
         const int n_tries = packed_forward_tries(const_cast<radon_geometry*>(g), dt, batch, cfg, f16w, tries);
         std::string why;
         for (int i = 0; i < n_tries; ++i) {
-            const radon_launch_config c = packed_forward_config(cfg, dt, tries[i].views);
+            const radon_launch_config c = packed_forward_config(cfg, dt, tries[i]);
             if (i == 0) {
                 cudaError_t e = launch_pack_images(in, ws, g->n, batch, dt, s);
                 if (e != cudaSuccess) return cuda_fail(e, "pack launch");
@@ -513,7 +524,7 @@ radon_status radon_forward_images_per_cta(const radon_geometry* g, radon_dtype d
     PackedTry tries[kMaxPackedTries];
     const int n_tries = packed_forward_tries(const_cast<radon_geometry*>(g), dtype, batch, config, f16w, tries);
     for (int i = 0; i < n_tries; ++i) {
-        const radon_launch_config c = packed_forward_config(config, dtype, tries[i].views);
+        const radon_launch_config c = packed_forward_config(config, dtype, tries[i]);
         PackedFwdShape sh;
         std::string why;
         if (packed_forward_shape(const_cast<radon_geometry*>(g), dtype, batch, &c, f16w, tries[i].lanes, &sh, &why) ==

@@ -145,12 +145,13 @@ struct PackedFwdShape {
 radon_status packed_forward_shape(radon_geometry* g, radon_dtype dt, int batch, const radon_launch_config* cfg,
                                   bool fp16_weights, int lanes, PackedFwdShape* out, std::string* why);
 
-// radon_api.cpp: the packed forward's shapes to try for a call, in order (views per CTA, lanes per ray); the
-// number of them.  A caller's views per CTA is the only one.  Otherwise one lane per ray over 8, 4, 2 and 1
-// views, then two lanes (narrower bands) where none fits -- but a batch of one texel group whose CTAs of
-// 8 views would not fill the GPU first tries two lanes over 4 views.
+// radon_api.cpp: the packed forward's shapes to try for a call, in order (views per CTA, lanes per ray, images
+// per CTA or 0 for the default); the number of them.  A caller's views per CTA is the only one.  Otherwise one
+// lane per ray over 8, 4, 2 and 1 views, then two lanes (narrower bands) where none fits -- but a batch of
+// one texel group whose CTAs of 8 views would not fill the GPU first tries two lanes over 4 views, and a pair
+// of groups that leaves an SM one CTA first tries single groups.
 struct PackedTry {
-    int views, lanes;
+    int views, lanes, images;
 };
 constexpr int kMaxPackedTries = 9;
 int packed_forward_tries(radon_geometry* g, radon_dtype dt, int batch, const radon_launch_config* cfg, bool fp16_weights,

@@ -85,7 +85,7 @@ extern "C" RADON_API radon_status radon_forward_static_scratch(const radon_geome
     const int n_tries = packed_forward_tries(const_cast<radon_geometry*>(geometry), dtype, batch, nullptr, false, tries);
     std::string why;
     for (int i = 0; i < n_tries; ++i) {
-        radon_launch_config c = {RADON_ALGO_TILED, tries[i].views, 0, 0, 0, 0, 0};
+        radon_launch_config c = {RADON_ALGO_TILED, tries[i].views, 0, tries[i].images, 0, 0, 0};
         st = launch_forward_packed(const_cast<radon_geometry*>(geometry), scratch, sino, dtype, batch, &c,
                                    identity_epilogue(), s, &why, tries[i].lanes);
         if (st == RADON_OK) {

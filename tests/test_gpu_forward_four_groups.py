@@ -51,7 +51,7 @@ def test_four_groups_match_the_oracle(case, dtype):
 def test_the_query_reports_four_groups():
     """Four groups where their CTAs fill the GPU: at least 300 of them, here 27 per four groups of images."""
     g, _ = make("parallel_n64_full")
-    for dtype, batch, images in ((torch.float16, 24, 16), (torch.float16, 32, 16), (torch.float16, 352, 16),
+    for dtype, batch, images in ((torch.float16, 24, 8), (torch.float16, 32, 8), (torch.float16, 352, 16),
                                  (torch.float16, 353, 32), (torch.bfloat16, 384, 32), (torch.float32, 16, 4),
                                  (torch.float32, 32, 4), (torch.float32, 176, 4), (torch.float32, 177, 16),
                                  (torch.float32, 192, 16)):

@@ -40,3 +40,22 @@ def test_thin_grids(args, dtype):
         one = forward_raw(g, x, launch_config("tiled", views_per_cta=8))
         assert (rel_l2(to_np(one), ref) <= TOL_F32) if dtype == torch.float32 else within_16(to_np(one), ref, dtype)
         assert L.radon_get_device_error(stream) == L.RADON_OK
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16], ids=["f16", "bf16"])
+@pytest.mark.parametrize("args,images", [
+    (dict(kind="parallel", n=64, angles=uniform_angles(64, math.pi), det_count=91), 8),        # fewer CTAs than SMs
+    (dict(kind="parallel", n=300, angles=uniform_angles(48, math.pi), det_count=425), 8),      # wide bands
+    (dict(kind="parallel", n=96, angles=uniform_angles(500, math.pi), det_count=137), 16),
+], ids=["few", "wide", "pair"])
+def test_pairs_of_groups(args, images, dtype):
+    """16-bit batches of more than eight images pair their texel groups where two CTAs of pairs fit an SM and
+    fill it; single groups give the same bits at the same rows."""
+    a = dict(args)
+    g, og = Geometry(a.pop("kind"), **a), O.Geometry.from_args(args)
+    assert forward_images_per_cta(g, dtype, 13) == images
+    x = to_dev(np.random.default_rng(13).uniform(0.0, 1.0, (13, g.n, g.n)), dtype)
+    y = forward_raw(g, x)
+    assert within_16(to_np(y[::4]), O.forward(og, to_np(x[::4])), dtype)
+    single = launch_config(images_per_cta=8, rows_per_slab=16 if images == 8 else 14)
+    assert torch.equal(forward_raw(g, x, single), y)
