@@ -243,8 +243,10 @@ RADON_API size_t radon_forward_workspace_size(const radon_geometry* geometry, ra
  * this call: one texel group (8 for 16-bit storage, 4 for FP32), two groups whose images share each
  * sample's position, floor and weight evaluation (16 / 8), or four that share each texel row's weights (32
  * / 16).  By default 16-bit batches of more than 8 images take two groups and of more than 24 four (FP32
- * weights), FP32 batches of more than 16 images four and smaller ones one, where the bands fit; `config`'s images_per_cta chooses where it holds one of those
- * values.  Where no shape with one thread per ray fits a TMA box (sparse views with a detector wider
+ * weights), FP32 batches of more than 16 images four and smaller ones one -- where the bands leave two such
+ * CTAs room on an SM, the batch fills their groups and the CTAs fill the GPU, else fewer groups; `config`'s
+ * images_per_cta chooses where it holds one or two groups' images.  A batch of one group on few CTAs takes
+ * two threads per ray over four views.  Where no shape with one thread per ray fits a TMA box (sparse views with a detector wider
  * than the image) and `config` fixes no views per CTA, two threads share each ray (half the detectors
  * per CTA, one texel group).  *images = 0 when another kernel serves the call (one image under AUTO,
  * the PLAIN algorithm, a geometry no packed shape takes).  Host only (host-only geometries are
@@ -269,7 +271,7 @@ RADON_API radon_status radon_forward_ws(const radon_geometry* geometry, const vo
  * batch packed into one row per (group, view, detector), laid out [group][view][detector][row], a row
  * holding the group's images in the storage type (bg 16-bit values, or bg FP32 values and four
  * padding words).  Groups of bg = 8 images for batches of at most 8, 16 up to 16; above that 16 for
- * 16-bit storage when the geometry holds an adjoint weight table, else 32 where whole groups of 32
+ * 16-bit storage when a fan geometry holds an adjoint weight table, else 32 where whole groups of 32
  * cost less than groups of 16 (a 32-image CTA costs ~1.56x a 16-image one) and their staging fits
  * one CTA's shared memory, else 16.  Returns 0 for an invalid geometry, dtype or batch.
  */
@@ -316,7 +318,9 @@ RADON_API radon_status radon_forward_static_scratch(const radon_geometry* geomet
  * detectors in a view (rays denser than a pixel, e.g. near a fan's source) are marked and keep
  * computing their weights.  While a geometry holds its table, the packed adjoint of batches that run
  * 8- or 16-image groups reads the weights instead of evaluating them: the same nonzero products added
- * in the same order, so the same bits.
+ * in the same order, so the same bits.  A parallel beam's weights are cheaper to evaluate than to read
+ * (all rays of a view share one step): there only groups of 16 images with a sampling step of
+ * sqrt(2) * 2 / 3 or less read the table.
  *   - radon_geometry_adjoint_table_size: the table's device bytes, tiles x views x (128 pairs x 44
  *     + 4) (4.2 GB for 512^2 and 720 views); no allocation.
  *   - radon_geometry_build_adjoint_table: allocates the table on the geometry's device (which must be
