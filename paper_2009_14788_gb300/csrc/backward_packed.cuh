@@ -14,6 +14,7 @@
 //     window constant C of its candidate samples -- meet at a named barrier and gather: each thread
 //     owns two vertically neighbouring pixels; for every candidate ray of either pixel, each pixel's KW
 //     sample weights once for all BG images, then one FP32 FMA per image and pixel from one row of loads.
+// Parallel beams copy and re-base no ray rows: one re-based ray per view places a window's rays (BwdPPar).
 // Shared-memory addresses stay 32-bit (explicit ld/st.shared), and no index needs a division.
 // The row pitch of (BG + 4) words is an odd number of 16-byte units, so the 16-byte loads of eight
 // lanes that read eight consecutive detectors fall in eight different bank groups.
