@@ -224,9 +224,10 @@ int packed_forward_tries(radon_geometry* g, radon_dtype dt, int batch, const rad
         // One texel group on fewer than two CTAs per SM: each warp waits for its own loads, and twice the warps
         // over bands of half the views are faster (8 x 512^2 BF16, 60 views, 184 CTAs: 127 -> 104 us; 368
         // CTAs of 120 views: 178 against 183).  FP32 bands take twice the copies per image: only where
-        // not even one CTA per SM runs (4 x 128^2, 128 views, 96 CTAs: 33 -> 28 us; 184 CTAs: 157 against 174).
+        // not even one CTA per SM runs (4 x 128^2, 128 views, 96 CTAs: 33 -> 28 us; 3 x 256^2, 64 views, 108 CTAs
+        // 53 -> 41; 144 CTAs either way: 400^2, 60 views 78 -> 71, 381^2 fan 74 -> 81; 184 CTAs: 157 -> 174).
         const long long ctas = (long long)g->group_count[3] * ((g->D + sh.Dt - 1) / sh.Dt);
-        if (ctas < (dt == RADON_F32 ? 152 : 2 * 152)) out[n++] = PackedTry{4, 2, 0};
+        if (ctas < (dt == RADON_F32 ? 144 : 2 * 152)) out[n++] = PackedTry{4, 2, 0};
     }
     if (batch > bg && !f16w && c8.images_per_cta == 0 && c8.rows_per_slab == 0 &&
         packed_forward_shape(g, dt, batch, &c8, false, 1, &sh, &why) == RADON_OK && sh.NG == 2) {
