@@ -175,7 +175,7 @@ def _check_out(out: torch.Tensor, like: torch.Tensor, shape) -> torch.Tensor:
 
 def forward_workspace_bytes(geom: Geometry, dtype: torch.dtype, batch: int) -> int:
     """Bytes of the workspace the packed forward path uses (``radon_forward_workspace_size``)."""
-    return geom.lib.radon_forward_workspace_size(geom.handle, _DTYPES[dtype], batch)
+    return geom.lib.radon_forward_workspace_size(geom.handle, _DTYPES[dtype], int(batch))
 
 
 def forward_images_per_cta(geom: Geometry, dtype: torch.dtype, batch: int, config=None) -> int:
@@ -226,7 +226,7 @@ def forward_raw(geom: Geometry, x: torch.Tensor, config=None, out=None, workspac
 
 def backward_workspace_bytes(geom: Geometry, dtype: torch.dtype, batch: int) -> int:
     """Bytes of the workspace the packed adjoint path uses (``radon_backward_workspace_size``)."""
-    return geom.lib.radon_backward_workspace_size(geom.handle, _DTYPES[dtype], batch)
+    return geom.lib.radon_backward_workspace_size(geom.handle, _DTYPES[dtype], int(batch))
 
 
 def _workspace(workspace, need, device):
