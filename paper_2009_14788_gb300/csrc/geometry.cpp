@@ -183,9 +183,13 @@ radon_status build_geometry(radon_geometry* g) {
             // k' * dxh exact in FP32 for -M <= k' < nk + M: dxh keeps 24 - bits(nk + M) significant bits.
             // The margin M covers the adjoint's reference sample, the one nearest a 16-pixel tile's
             // centre, which may sit up to (tile half-diagonal + support) / h samples past a ray end.
+            // A parallel ray that misses the image may still place its neighbours' samples in a tile at the
+            // image's edge (the adjoint's one ray per view): from its foot point that tile is up to half a
+            // diagonal away, either way.
             const long margin = kSplitMarginPx * (long)std::ceil(1.0 / g->h) + 8;
+            const long reach = hit || g->fan ? nk : (long)std::ceil(0.75 * (g->n + 1) / g->h);
             int kbits = 1;
-            while (kbits < 24 && ((long)1 << kbits) < (long)nk + margin) ++kbits;
+            while (kbits < 24 && ((long)1 << kbits) < reach + margin) ++kbits;
             const int hbits = std::max(1, 24 - kbits);
             const double hx = round_bits(sx, hbits), hy = round_bits(sy, hbits);
             rt.dxh = (float)hx;
