@@ -169,10 +169,9 @@ radon_status build_adjoint_table(radon_geometry* g, std::string* why) {
     if (e == cudaSuccess) e = cudaMemset(vflag, 0, tv * sizeof(int));
     if (e == cudaSuccess) {
         const dim3 grid((unsigned)(tiles_x * tiles_x), (unsigned)((g->V + kViewsPerBlock - 1) / kViewsPerBlock));
-        const float ih2 = (float)(1.0 / (g->h * g->h));
         auto kern = g->fan ? (kw == 3 ? bwdp_table_kernel<3, false> : bwdp_table_kernel<6, false>)
                            : (kw == 3 ? bwdp_table_kernel<3, true> : bwdp_table_kernel<6, true>);
-        kern<<<grid, kBwdTabPairs>>>(g->d_ray, g->d_view, g->n, g->V, g->D, ih2, wd, tiles_x, kViewsPerBlock, w, w5, la,
+        kern<<<grid, kBwdTabPairs>>>(g->d_ray, g->d_view, g->n, g->V, g->D, bwdp_lattice(g), wd, tiles_x, kViewsPerBlock, w, w5, la,
                                      vflag, over);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaDeviceSynchronize();

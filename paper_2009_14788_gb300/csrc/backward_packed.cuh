@@ -82,13 +82,19 @@ __host__ __device__ inline BwdPSmem bwdp_smem(int wd, int stages, bool rays) {
     return m;
 }
 
+// Scales of a geometry: 1 / step^2 (every ray's step has length h); for parallel beams also 1 / det_spacing^2 and
+// det_spacing / step in two parts.
+struct BwdPLattice {
+    float ih2, id2, nh, nl;
+};
+
 struct BwdPArgs {
     const ViewF* views;
     const RayT* rays;  // the ray table (parallel beams)
     void* img;
     int n, V, D, B;
     float h;           // output scale (the step; 1 for the interpolating backprojector)
-    float ih2;         // 1 / step^2 (every ray's step has length h)
+    BwdPLattice lattice;
     int wd;            // detector window per view (rows copied per view)
     int stages;        // ring depth (2..kBwdPMaxStages)
     int tiles_x;
@@ -166,68 +172,65 @@ __device__ __forceinline__ float bwdp_weight(float px, float py, float s, const 
     return w;
 }
 
-// Parallel beams: every ray of a view has the same step and the rays' sample lattices line up (sample k of ray
-// d + 1 is sample k of ray d moved by det_spacing * n, n the detector axis), so one re-based ray per view and
-// tile places them all.  A view's record, for tile-local pixels p and window rays l = 0, 1, ...:
-//   t = ax px + ay py + a0               window-relative detector coordinate
+// Parallel beams: one re-based ray per view and tile places them all (bwd_tile_ray).  A view's record, for pixels p
+// about the tile's centre and window rays l = 0, 1, ...:
+//   t = (n . p) / det_spacing^2 + t0     window-relative detector coordinate
 //   s = b . p + c, b = step / h^2        its nearest integer is the first candidate sample (the same
 //                                        lattice index on every ray; c holds the window's half width)
-//   A + k step + (l - l0) n - p          sample k of window ray l relative to the pixel, n = q (ax, ay)
-// The reference ray l0 is the one nearest the window's middle, so the error of n is multiplied little.  A
-// candidate ray then costs a pixel two additions and its samples' tents instead of a record's two shared
+//   (l - l0) n + s step - p + A          sample s of window ray l relative to the pixel
+// A candidate ray then costs a pixel two additions and its samples' tents instead of a record's two shared
 // loads, its first sample and its offset from the pixel, and no ray rows are copied or re-based (us, ray
 // records -> one ray per view, FP32, 512 views of 512^2: 8 images 898 -> 675, 16 images 1056 -> 854, 32
 // images 1581 -> 1286; 4 x 64^2, 64 views: 42 -> 30).
 struct BwdPPar {
-    float ax, ay, a0, c;
+    float nx, ny, t0, c;
     float Ax, Ay, sx, sy;
-    float q, l0;
+    float l0;
 };
 
-__device__ __forceinline__ BwdPPar bwdp_par_view(const ViewF vf, const RayT* __restrict__ rays, int v, int D, int wd,
-                                                 int dlo, int ti, int tj, float ih2) {
-    const int dref = min(max(dlo + (wd >> 1), 0), D - 1);
-    const float4 A = bwd_ray_pos_rec(rays[(long long)v * D + dref], true, ti, tj, ih2);
-    const float bx = A.z * ih2, by = A.w * ih2;
+__device__ __forceinline__ BwdPPar bwdp_par_view(const ViewF vf, const RayT* __restrict__ rays, int v, int D, int n,
+                                                 int dlo, int ti, int tj, const BwdPLattice g) {
+    const BwdTileRay A = bwd_tile_ray(vf, rays + (long long)v * D, D, n, ti, tj, g.ih2, g.nh, g.nl);
+    const float bx = A.sx * g.ih2, by = A.sy * g.ih2;
     BwdPPar w;
-    w.ax = vf.ax;
-    w.ay = vf.ay;
-    w.a0 = bwd_det_coord(vf, (float)tj, (float)ti) - (float)dlo;
-    w.c = (-fmaf(A.x, bx, A.y * by) - fmaf(fabsf(A.z) + fabsf(A.w), ih2, 1e-4f)) + 0.5f;
-    w.Ax = A.x;
-    w.Ay = A.y;
-    w.sx = A.z;
-    w.sy = A.w;
-    w.q = 1.0f / fmaf(vf.ax, vf.ax, vf.ay * vf.ay);
-    w.l0 = (float)(dref - dlo);
+    w.nx = A.nx;
+    w.ny = A.ny;
+    w.t0 = bwd_det_affine(vf, (float)tj + kBwdMid, (float)ti + kBwdMid) - (float)dlo;
+    w.c = (-fmaf(A.ax, bx, A.ay * by) - fmaf(fabsf(A.sx) + fabsf(A.sy), g.ih2, 1e-4f)) + 0.5f;
+    w.Ax = A.ax;
+    w.Ay = A.ay;
+    w.sx = A.sx;
+    w.sy = A.sy;
+    w.l0 = (float)(A.d - dlo);
     return w;
 }
 
 // A pixel pair's walk over the window rays of one view: [la, lb] the union of the pixels' candidates,
-// (rx, ry) each pixel's first candidate sample on ray la, (nx, ny) the move to the next ray.
+// (rx, ry) each pixel's first candidate sample on ray la.
 struct BwdPWalk {
     int la, lb;
-    float rx[2], ry[2], nx, ny;
+    float rx[2], ry[2];
 };
 
-__device__ __forceinline__ BwdPWalk bwdp_par_walk(const BwdPPar w, float r, float px, float py0, float ih2, int wd) {
+// The pair's upper pixel at (px, py0) about the tile's centre.
+__device__ __forceinline__ BwdPWalk bwdp_par_walk(const BwdPPar w, float r, float px, float py0, const BwdPLattice g,
+                                                  int wd) {
     constexpr float kMagic = 12582912.0f;   // 1.5 * 2^23: x + kMagic rounds x to the nearest integer
     BwdPWalk k;
-    const float t0 = fmaf(w.ax, px, fmaf(w.ay, py0, w.a0)), t1 = t0 + w.ay;
+    const float t0 = fmaf(fmaf(w.nx, px, w.ny * py0), g.id2, w.t0), t1 = fmaf(w.ny, g.id2, t0);
     const float fa = ceilf(fmaxf(fminf(t0, t1) - r, 0.0f));
     k.la = (int)fa;
     k.lb = __float2int_rd(fminf(fmaxf(t0, t1) + r, (float)(wd - 1)));
-    k.nx = w.ax * w.q;
-    k.ny = w.ay * w.q;
-    const float bx = w.sx * ih2, by = w.sy * ih2;
+    const float bx = w.sx * g.ih2, by = w.sy * g.ih2;
     const float s0 = fmaf(bx, px, fmaf(by, py0, w.c));
     const float ka0 = (s0 + kMagic) - kMagic, ka1 = ((s0 + by) + kMagic) - kMagic;
     const float l = fa - w.l0;
-    const float ux = fmaf(l, k.nx, w.Ax - px), uy0 = fmaf(l, k.ny, w.Ay - py0), uy1 = fmaf(l, k.ny, w.Ay - (py0 + 1.0f));
-    k.rx[0] = fmaf(ka0, w.sx, ux);
-    k.ry[0] = fmaf(ka0, w.sy, uy0);
-    k.rx[1] = fmaf(ka1, w.sx, ux);
-    k.ry[1] = fmaf(ka1, w.sy, uy1);
+    // the terms of up to eleven pixels first, cancelling to about one, then the sample's own small offset
+    const float ux = fmaf(l, w.nx, -px), uy0 = fmaf(l, w.ny, -py0), uy1 = fmaf(l, w.ny, -(py0 + 1.0f));
+    k.rx[0] = fmaf(ka0, w.sx, ux) + w.Ax;
+    k.ry[0] = fmaf(ka0, w.sy, uy0) + w.Ay;
+    k.rx[1] = fmaf(ka1, w.sx, ux) + w.Ax;
+    k.ry[1] = fmaf(ka1, w.sy, uy1) + w.Ay;
     return k;
 }
 
@@ -307,9 +310,9 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
     float* r_c = reinterpret_cast<float*>(smem + 256);            // [stages][views]
     ViewF* view_c = reinterpret_cast<ViewF*>(smem + 512);         // [stages][views]
     int* fly_c = reinterpret_cast<int*>(smem + 320);              // [stages]: the chunk takes weights on the fly
-    float2* par_c = reinterpret_cast<float2*>(smem + 352);        // [stages][views] parallel: (q, l0)
+    float* par_c = reinterpret_cast<float*>(smem + 352);          // [stages][views] parallel: l0
     static_assert(kBwdPMaxStages * kBwdPViews * 4 <= 64 && kBwdPMaxStages * 4 <= 32 &&
-                      352 + kBwdPMaxStages * kBwdPViews * 8 <= 512 &&
+                      352 + kBwdPMaxStages * kBwdPViews * 4 <= 512 &&
                       512 + kBwdPMaxStages * kBwdPViews * 32 <= kBwdPHeader && sizeof(ViewF) == 32,
                   "ring header overflows its slots");
     const int S = a.stages;
@@ -340,7 +343,7 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
         while (ok && c < nchunks) {
             const int vlane = c * kBwdPViews + lane;
             ViewF vf{};
-            float2 par = make_float2(0.0f, 0.0f);
+            float par = 0.0f;
             int dlo = 0;
             float r = 0.0f;
             unsigned flagged = 0;
@@ -352,16 +355,16 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
                 const float thi = floorf(bwdp_tile_tmax(vf, ti, tj, a.n) + r);
                 if (fminf(thi, (float)(a.D - 1)) > (float)(dlo + a.wd - 1)) record_device_error(a.err, RADON_ERR_DEVICE_BOUNDS);
                 if constexpr (PAR) {   // the first eight words of the view's record in the place of its map
-                    const BwdPPar w = bwdp_par_view(vf, a.rays, vlane, a.D, a.wd, dlo, ti, tj, a.ih2);
-                    vf.ax = w.ax;
-                    vf.ay = w.ay;
-                    vf.a0 = w.a0;
+                    const BwdPPar w = bwdp_par_view(vf, a.rays, vlane, a.D, a.n, dlo, ti, tj, a.lattice);
+                    vf.ax = w.nx;
+                    vf.ay = w.ny;
+                    vf.a0 = w.t0;
                     vf.bx = w.c;
                     vf.by = w.Ax;
                     vf.b0 = w.Ay;
                     vf.major = __float_as_int(w.sx);
                     vf.pad = __float_as_int(w.sy);
-                    par = make_float2(w.q, w.l0);
+                    par = w.l0;
                 }
             }
             // weights on the fly: always without a table, with one only where some pair overflows
@@ -514,7 +517,7 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
                     ray.dxl = hi.z;
                     ray.dyl = hi.w;
                     float4 A, Bc;
-                    bwdp_rebase(ray, d >= 0 && d < a.D, ti, tj, a.ih2, &A, &Bc);
+                    bwdp_rebase(ray, d >= 0 && d < a.D, ti, tj, a.lattice.ih2, &A, &Bc);
                     sts4(rec, A);
                     sts1(rec + 16, Bc.z);
                 }
@@ -674,12 +677,12 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
                 const float r = r_c[st * kBwdPViews + vl];
                 if constexpr (PAR) {
                     if (!tabbed) {
-                        const float2 ex = lds2(par_a + (uint32_t)(st * kBwdPViews + vl) * 8u);
-                        const BwdPPar view = {v01.x, v01.y, v01.z, v01.w, v23.x, v23.y, v23.z, v23.w, ex.x, ex.y};
-                        BwdPWalk k = bwdp_par_walk(view, r, px, py0, a.ih2, a.wd);
+                        const BwdPPar view = {v01.x, v01.y, v01.z, v01.w, v23.x, v23.y, v23.z, v23.w,
+                                              lds1(par_a + (uint32_t)(st * kBwdPViews + vl) * 4u)};
+                        BwdPWalk k = bwdp_par_walk(view, r, px - kBwdMid, py0 - kBwdMid, a.lattice, a.wd);
                         uint32_t ya = yv + (uint32_t)k.la * PITCH;
                         if constexpr (kPaired) {
-                            const f32x2 step = f2_pack(view.sx, view.sy), next = f2_pack(k.nx, k.ny);
+                            const f32x2 step = f2_pack(view.sx, view.sy), next = f2_pack(view.nx, view.ny);
                             f32x2 r2[PX] = {f2_pack(k.rx[0], k.ry[0]), f2_pack(k.rx[1], k.ry[1])};
                             for (int dl = k.la; dl <= k.lb; ++dl, ya += PITCH) {
                                 float w[PX];
@@ -696,8 +699,8 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
 #pragma unroll
                                 for (int x = 0; x < PX; ++x) {
                                     w[x] = bwdp_tents<KW>(k.rx[x], k.ry[x], view.sx, view.sy);
-                                    k.rx[x] += k.nx;
-                                    k.ry[x] += k.ny;
+                                    k.rx[x] += view.nx;
+                                    k.ry[x] += view.ny;
                                 }
                                 add_row(ya, w);
                             }
@@ -721,7 +724,7 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
                     uint32_t ya = yv + (uint32_t)la * PITCH;
                     for (int dl = la; dl <= lb; ++dl, ra += 32u, ya += PITCH) {
                         const float4 A = lds4(ra);
-                        const float bx = A.z * a.ih2, by = A.w * a.ih2;   // as re-basing computed them
+                        const float bx = A.z * a.lattice.ih2, by = A.w * a.lattice.ih2;   // as re-basing computed them
                         const float s0 = fmaf(px, bx, fmaf(py0, by, lds1(ra + 16)));
                         float w[PX];
                         w[0] = bwdp_weight<KW>(px, py0, s0, A);
@@ -757,7 +760,8 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
 template <int KW, bool PAR>
 __global__ void __launch_bounds__(kBwdTabPairs) bwdp_table_kernel(const RayT* __restrict__ rays,
                                                                  const ViewF* __restrict__ views, int n, int V, int D,
-                                                                 float ih2, int wd, int tiles_x, int views_per_block,
+                                                                 const BwdPLattice lattice, int wd, int tiles_x,
+                                                                 int views_per_block,
                                                                  float4* __restrict__ tab_w, float2* __restrict__ tab_w5,
                                                                  int* __restrict__ tab_la, int* __restrict__ tab_vflag,
                                                                  unsigned long long* overflow) {
@@ -785,8 +789,8 @@ __global__ void __launch_bounds__(kBwdTabPairs) bwdp_table_kernel(const RayT* __
         BwdPPar view{};
         BwdPWalk walk{};
         if constexpr (PAR) {
-            view = bwdp_par_view(vf, rays, v, D, wd, dlo, ti, tj, ih2);
-            walk = bwdp_par_walk(view, r, px, py0, ih2, wd);
+            view = bwdp_par_view(vf, rays, v, D, n, dlo, ti, tj, lattice);
+            walk = bwdp_par_walk(view, r, px - kBwdMid, py0 - kBwdMid, lattice, wd);
             la = walk.la;
             lb = walk.lb;
         }
@@ -794,10 +798,10 @@ __global__ void __launch_bounds__(kBwdTabPairs) bwdp_table_kernel(const RayT* __
             if constexpr (PAR) {   // the gather's steps from ray la
                 BwdPWalk k = walk;
                 for (int l = la; l < dl; ++l) {
-                    k.rx[0] += k.nx;
-                    k.ry[0] += k.ny;
-                    k.rx[1] += k.nx;
-                    k.ry[1] += k.ny;
+                    k.rx[0] += view.nx;
+                    k.ry[0] += view.ny;
+                    k.rx[1] += view.nx;
+                    k.ry[1] += view.ny;
                 }
                 *w0 = bwdp_tents<KW>(k.rx[0], k.ry[0], view.sx, view.sy);
                 *w1 = bwdp_tents<KW>(k.rx[1], k.ry[1], view.sx, view.sy);
@@ -808,7 +812,7 @@ __global__ void __launch_bounds__(kBwdTabPairs) bwdp_table_kernel(const RayT* __
             RayT ray{0, 0, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
             if (valid) ray = rays[(long long)v * D + d];
             float4 A, Bc;
-            bwdp_rebase(ray, valid, ti, tj, ih2, &A, &Bc);
+            bwdp_rebase(ray, valid, ti, tj, lattice.ih2, &A, &Bc);
             const float s0 = fmaf(px, Bc.x, fmaf(py0, Bc.y, Bc.z));
             *w0 = bwdp_weight<KW>(px, py0, s0, A);
             *w1 = bwdp_weight<KW>(px, py0 + 1.0f, s0 + Bc.y, A);
@@ -854,6 +858,12 @@ inline size_t bwdp_plan(int wd, bool rays, int* stages) {
     while (S > 2 && bwdp_smem<T, BG>(wd, S, rays).total > budget) --S;
     *stages = S;
     return bwdp_smem<T, BG>(wd, S, rays).total;
+}
+
+inline BwdPLattice bwdp_lattice(const radon_geometry* g) {
+    const double c = g->ds / g->h;
+    const float nh = (float)c;
+    return BwdPLattice{(float)(1.0 / (g->h * g->h)), (float)(1.0 / (g->ds * g->ds)), nh, (float)(c - nh)};
 }
 
 // Whether the exact adjoint of groups of bg images reads the geometry's weight table.
@@ -921,7 +931,7 @@ radon_status launch_backward_packed_t(const radon_geometry* g, const void* packe
     a.D = g->D;
     a.B = batch;
     a.h = kw == 0 ? 1.0f : (float)g->h;   // the interpolating backprojector's sum carries no step factor
-    a.ih2 = (float)(1.0 / (g->h * g->h));
+    a.lattice = bwdp_lattice(g);
     a.wd = wd;
     a.stages = stages;
     a.tiles_x = (g->n + kBwdTile - 1) / kBwdTile;
