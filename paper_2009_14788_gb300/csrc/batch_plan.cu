@@ -55,6 +55,7 @@ struct Unit {
     long long q_off;   // forward: first texel of this unit's packed image (row frame; transposed follows)
     int n, V, D;
     float h, ih2;
+    float nh, nl;      // adjoint, parallel beam: det_spacing / step in two parts
     int wd;            // adjoint: detector window of a 16 x 16 tile
     int cfg;           // forward: views per ray block; adjoint: views per chunk
     int lanes;         // forward: lanes per ray (1 or 4)
@@ -305,16 +306,18 @@ __global__ void __launch_bounds__(kPlanThreads, 6) single_forward_kernel(const U
 
 // ------------------------------------------------------------------------------------- adjoint
 
-// One view of a parallel-beam chunk, as the gather of a tile reads it (tile-local pixel p):
+// One view of a parallel-beam chunk, as the gather of a tile reads it (pixel p about the tile's centre):
 //   t' = ax px + ay py + a0   window-relative detector coordinate, shifted so that its nearest integer is
 //                             the first candidate ray (for the counted gather; unshifted for the loop)
 //   s' = bx px + by py + c    the same along the rays: its nearest integer is the first candidate sample
-//   (Ax, Ay), (sx, sy), (nx, ny)   window ray 0's reference sample relative to the tile, the step along a
+//   (Ax, Ay), (sx, sy), (nx, ny)   the reference sample of window ray l0 (bwd_tile_ray), the step along a
 //                             ray and the offset from one ray's samples to the next ray's
+//   l0m = l0 + 1.5 * 2^23     taken off a rounded coordinate, it leaves the ray's place from l0 (exact)
 struct alignas(16) AdjView {
     float ax, ay, a0, c;
     float Ax, Ay, sx, sy;
     float nx, ny, bx, by;
+    float l0m, pad[3];
 };
 
 struct AdjShared {
@@ -440,8 +443,8 @@ __device__ void plan_adjoint_tile(const Unit& u, int tile, const AdjBuffers& b, 
 
 // Parallel beams: every ray of a view has the same direction and the rays' sample lattices line up
 // (sample k of ray d sits at m_d + k h u with m_d = s_d n, so sample k of ray d + 1 is sample k of
-// ray d moved by det_spacing * n).  So the CTA re-bases one ray per view -- the window's first --
-// and stages only the window's sinogram values; each pixel finds its first candidate sample ka once
+// ray d moved by det_spacing * n).  So the CTA re-bases one ray per view (bwd_tile_ray) and stages
+// only the window's sinogram values; each pixel finds its first candidate sample ka once
 // per view (the same lattice index on every ray) and steps from one candidate ray to the next by
 // det_spacing * n.  Every lattice point within a pixel's 2 x 2 support lies inside the support box,
 // so it is a sample of its ray whenever the ray exists; rays outside the detector have zero values.
@@ -468,8 +471,8 @@ __device__ void plan_adjoint_tile_parallel(const Unit& u, int tile, const AdjBuf
     // pixels past the image's edge repeat the edge's: every coordinate stays within the tile's corners
     const int xe = min(kBwdTile - 1, u.n - 1 - tj), ye = min(kBwdTile - 1, u.n - 1 - ti);
     const int pe = PX == 2 ? pi0 : pi0 & ~1;     // the pair's upper row
-    const float px = (float)min(pj, xe), py0 = (float)min(pe, ye);
-    const float py1 = PX == 1 && pe == pi0 ? py0 : (float)min(pe + 1, ye);
+    const float px = (float)min(pj, xe) - kBwdMid, py0 = (float)min(pe, ye) - kBwdMid;
+    const float py1 = PX == 1 && pe == pi0 ? py0 : (float)min(pe + 1, ye) - kBwdMid;
     const f32x2 np0 = f2_pack(-px, -py0), np1 = f2_pack(-px, -py1);
     const float dy = py1 - py0;
     const T* y = static_cast<const T*>(u.in);
@@ -488,29 +491,26 @@ __device__ void plan_adjoint_tile_parallel(const Unit& u, int tile, const AdjBuf
             // every pixel's candidates [ceil(t - r), floor(t + r)] within the detector must lie in the
             // staged window (the tile's largest t is at a corner); a miss is recorded, not overrun
             const float x1 = (float)(tj + xe), y1 = (float)(ti + ye);
-            const float t00 = bwd_det_coord(vf, (float)tj, (float)ti), t10 = bwd_det_coord(vf, x1, (float)ti);
-            const float t01 = bwd_det_coord(vf, (float)tj, y1), t11 = bwd_det_coord(vf, x1, y1);
+            const float t00 = bwd_det_affine(vf, (float)tj, (float)ti), t10 = bwd_det_affine(vf, x1, (float)ti);
+            const float t01 = bwd_det_affine(vf, (float)tj, y1), t11 = bwd_det_affine(vf, x1, y1);
             const float tmax = fmaxf(fmaxf(t00, t10), fmaxf(t01, t11)), tmin = fminf(fminf(t00, t10), fminf(t01, t11));
             if (fminf(floorf(tmax + r), (float)(u.D - 1)) > (float)(dlo + wd - 1)) record_device_error(err, RADON_ERR_DEVICE_BOUNDS);
-            // every ray keeps its line in the table (a ray missing the image included)
-            const int dref = min(max(dlo, 0), u.D - 1);
-            const float4 A = bwd_ray_pos_rec(u.rays[(long long)(c0 + tid) * u.D + dref], true, ti, tj, u.ih2);
-            // det_spacing * n = (ax, ay) / (ax^2 + ay^2): the map t = (n.P) / det_spacing + const
-            const float q = 1.0f / fmaf(vf.ax, vf.ax, vf.ay * vf.ay);
-            const float sh = (float)(dlo - dref);
+            const BwdTileRay A = bwd_tile_ray(vf, u.rays + (long long)(c0 + tid) * u.D, u.D, u.n, ti, tj, u.ih2, u.nh, u.nl);
             AdjView w;
-            w.nx = vf.ax * q;
-            w.ny = vf.ay * q;
-            w.bx = A.z * u.ih2;
-            w.by = A.w * u.ih2;
-            w.c = -fmaf(A.x, w.bx, A.y * w.by) - fmaf(fabsf(A.z) + fabsf(A.w), u.ih2, 1e-4f) + 0.5f;
-            w.Ax = fmaf(sh, w.nx, A.x);
-            w.Ay = fmaf(sh, w.ny, A.y);
-            w.sx = A.z;
-            w.sy = A.w;
+            w.nx = A.nx;
+            w.ny = A.ny;
+            w.bx = A.sx * u.ih2;
+            w.by = A.sy * u.ih2;
+            w.c = -fmaf(A.ax, w.bx, A.ay * w.by) - fmaf(fabsf(A.sx) + fabsf(A.sy), u.ih2, 1e-4f) + 0.5f;
+            w.Ax = A.ax;
+            w.Ay = A.ay;
+            w.sx = A.sx;
+            w.sy = A.sy;
+            w.l0m = (float)(A.d - dlo) + kMagic;
             w.ax = vf.ax;
             w.ay = vf.ay;
-            w.a0 = t00 - (float)dlo;   // the tile's first pixel; r's margin covers the rounding of t00
+            // the tile's centre; r's margin covers the coordinate's rounding
+            w.a0 = bwd_det_affine(vf, (float)tj + kBwdMid, (float)ti + kBwdMid) - (float)dlo;
             if (NC > 0) {
                 // the first candidates' nearest integers stay in [0, wd - 1] (0.05 covers the rounding of
                 // the per-pixel coordinates), so the NC rays lie within the staged values
@@ -539,6 +539,7 @@ __device__ void plan_adjoint_tile_parallel(const Unit& u, int tile, const AdjBuf
         uint32_t yb = ys_a - 4u * kMagicBits;    // the magic number's bits cancel modulo 2^32
         for (int vl = 0; vl < nv; ++vl, va += (uint32_t)sizeof(AdjView), yb += 4u * (uint32_t)wp) {
             const float4 v0 = lds4(va), v1 = lds4(va + 16), v2 = lds4(va + 32);
+            const float l0m = lds1(va + 48);
             const f32x2 A2 = f2_pack(v1.x, v1.y), st2 = f2_pack(v1.z, v1.w), dn2 = f2_pack(v2.x, v2.y);
             const float t0 = fmaf(v0.x, px, fmaf(v0.y, py0, v0.z)), t1 = fmaf(v0.y, dy, t0);
             const float s0 = fmaf(v2.z, px, fmaf(v2.w, py0, v0.w)), s1 = fmaf(v2.w, dy, s0);
@@ -557,13 +558,15 @@ __device__ void plan_adjoint_tile_parallel(const Unit& u, int tile, const AdjBuf
                 }
                 return w;
             };
-            auto first = [&](f32x2 np, float ka, float la) {   // sample ka of ray la, relative to the pixel
-                return f2_fma(f2_pack(ka, ka), st2, f2_fma(f2_pack(la, la), dn2, f2_add(A2, np)));
+            // sample ka of the ray l away from l0, relative to the pixel: the terms of up to eleven pixels first,
+            // cancelling to about one, then the sample's own small offset
+            auto first = [&](f32x2 np, float ka, float l) {
+                return f2_add(f2_fma(f2_pack(ka, ka), st2, f2_fma(f2_pack(l, l), dn2, np)), A2);
             };
             if constexpr (NC > 0) {
                 const float m0 = t0 + kMagic, m1 = t1 + kMagic;
-                [[maybe_unused]] f32x2 ra = first(np0, ka0, m0 - kMagic);
-                f32x2 rb = first(np1, ka1, m1 - kMagic);
+                [[maybe_unused]] f32x2 ra = first(np0, ka0, m0 - l0m);
+                f32x2 rb = first(np1, ka1, m1 - l0m);
                 const uint32_t ya = yb + 4u * __float_as_uint(m0), yc = yb + 4u * __float_as_uint(m1);
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
@@ -581,7 +584,7 @@ __device__ void plan_adjoint_tile_parallel(const Unit& u, int tile, const AdjBuf
                 auto loop = [&](f32x2 np, float t, float ka, float& acc) {
                     const float la = fmaxf(ceilf(t - r), 0.0f);
                     const int lb = __float2int_rd(fminf(t + r, wd_last));
-                    f32x2 r2 = first(np, ka, la);
+                    f32x2 r2 = first(np, ka, la - (l0m - kMagic));
                     for (int l = (int)la; l <= lb; ++l) {
                         acc = fmaf(weight(r2), b.ys[vl * wp + l], acc);
                         r2 = f2_add(r2, dn2);
@@ -787,6 +790,13 @@ cudaError_t staged_smem_attr(size_t smem) {
     return raise_smem_attr<staged_forward_kernel<T>>(smem);
 }
 
+void set_scales(Unit& u, const radon_geometry* g) {
+    const double c = g->ds / g->h;
+    u.ih2 = (float)(1.0 / (g->h * g->h));
+    u.nh = (float)c;
+    u.nl = (float)(c - u.nh);
+}
+
 Unit single_unit(const radon_geometry* g, const void* in, void* out, int cfg) {
     Unit u;
     u.in = in;
@@ -799,7 +809,7 @@ Unit single_unit(const radon_geometry* g, const void* in, void* out, int cfg) {
     u.V = g->V;
     u.D = g->D;
     u.h = (float)g->h;
-    u.ih2 = (float)(1.0 / (g->h * g->h));
+    set_scales(u, g);
     u.wd = g->bwd_window + 2;
     u.cfg = cfg;
     u.lanes = kSingleForwardLanes;
@@ -1294,7 +1304,7 @@ extern "C" RADON_API radon_status radon_batch_plan_create(const radon_item* item
             u.V = g->V;
             u.D = g->D;
             u.h = (float)g->h;
-            u.ih2 = (float)(1.0 / (g->h * g->h));
+            set_scales(u, g);
             u.wd = g->bwd_window + 2;
             u.fan = g->fan;
             u.cand3 = direction == 1 ? three_candidates(g) : 0;

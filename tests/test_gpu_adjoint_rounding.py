@@ -34,7 +34,7 @@ def test_rounding_of_the_rays_places(n, views, det, spacing, step):
     g, og = _make(n, np.arange(views) * (math.pi / views), det, spacing, step)
     y = np.random.default_rng(n + views).normal(size=(1, views, det)).astype(np.float32)
     ref = O.adjoint(og, y)
-    for batch in (3, 16, 32):
+    for batch in (1, 3, 16, 32):
         got = to_np(backward_raw(g, to_dev(np.repeat(y, batch, 0))))
         assert (got == got[:1]).all()
         assert rel_l2(got[:1], ref) <= GATE, batch
@@ -50,7 +50,7 @@ def test_tiles_of_a_few_pixels_at_the_images_edge(n):
     y = np.random.default_rng(n).normal(size=(1, len(angles), 1451)).astype(np.float32)
     ref = O.adjoint(og, y)[0]
     edge = n // 16 * 16
-    for batch in (3, 16, 32):
+    for batch in (1, 3, 16, 32):
         got = to_np(backward_raw(g, to_dev(np.repeat(y, batch, 0))))[batch - 1]
         assert rel_l2(got[edge:], ref[edge:]) <= GATE, batch
         assert rel_l2(got[:, edge:], ref[:, edge:]) <= GATE, batch
