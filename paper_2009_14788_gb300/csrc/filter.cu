@@ -27,9 +27,11 @@ constexpr int kFilterKinds = 5;
 constexpr int kFilterThreads = 256;
 constexpr int kFilterOut = 8;    // outputs per thread
 constexpr int kLongOut = 4;      // consecutive outputs per thread of the kernel for long rows
-// Taps nearer than this also add their lo part.  Every kernel here falls off like 1 / m^2, so the rounding
-// errors of all farther taps together stay below 2^-25 / (64 pi^2) = 5e-11 of the largest input, under
-// 1e-7 of a result a thousand times smaller (FP32 sums of a few hundred terms carry that much).
+// Taps nearer than this also add their lo part.  Every kernel here falls off like 1 / m^2: all farther taps
+// together are at most 2.5e-3 (cosine; 1.6e-3 the others), so leaving their rounding (up to 2^-24 each) moves
+// a result by at most 1.5e-10 of the largest input, a twenty-fifth of what one rounding of the sum at its
+// largest moves it (2^-25 / 8).  With every lo part the errors against 64 bits are the same in three digits
+// (91 .. 4000 bins, all windows, smooth and random rows), and 4000 bins take 655 instead of 309 us.
 constexpr int kFilterNear = 64;
 
 using cd = std::complex<double>;
@@ -158,8 +160,8 @@ __host__ __device__ inline FilterPlan filter_plan(int D) {
 // (fma.rn.f32x2: half the instructions), so an output's taps are needed as pairs at even and at odd
 // offsets: the reversed taps lie in shared memory twice, the second copy shifted by one, and both
 // windows slide in registers, one 16-byte load of each per four bins.  With Ram-Lak the zero taps are
-// left out.  512 views of 725 bins, FP32: 77 us with one bin per scalar FMA, both tap parts and the
-// zeros; 11 us so (a whole filtered backprojection 416 -> 351 us).
+// left out.  512 views of 725 bins, FP32: 73 us with one bin per scalar FMA, both tap parts and the
+// zeros; 24 us so (30 us under the other windows; 500 views of 4000 bins 2078 -> 306 us).
 template <typename T, bool HALF>
 __global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const T* __restrict__ in, T* __restrict__ out,
                                                                      const float2* __restrict__ taps, int D,
@@ -244,6 +246,37 @@ __global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const T* __
                     d1 = dd.y;
                 }
             };
+            // the same from the last bins to the first
+            auto conv_back = [&](const float* xi, const float* e, const float* d, int n) {
+                ulonglong2 ee = *reinterpret_cast<const ulonglong2*>(e + n - 4), em = *reinterpret_cast<const ulonglong2*>(e + n - 8);
+                ulonglong2 dd = *reinterpret_cast<const ulonglong2*>(d + n - 4), dm = *reinterpret_cast<const ulonglong2*>(d + n - 8);
+#pragma unroll 3
+                for (int i = n - 4; i >= 0; i -= 4) {
+                    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(xi + i);
+                    const ulonglong2 eb = *reinterpret_cast<const ulonglong2*>(e + i - 8);
+                    const ulonglong2 db = *reinterpret_cast<const ulonglong2*>(d + i - 8);
+                    acc[0] = f2_fma(v.y, ee.y, acc[0]);
+                    acc[1] = f2_fma(v.y, dd.y, acc[1]);
+                    acc[2] = f2_fma(v.y, ee.x, acc[2]);
+                    acc[3] = f2_fma(v.y, dd.x, acc[3]);
+                    acc[4] = f2_fma(v.y, em.y, acc[4]);
+                    acc[5] = f2_fma(v.y, dm.y, acc[5]);
+                    acc[6] = f2_fma(v.y, em.x, acc[6]);
+                    acc[7] = f2_fma(v.y, dm.x, acc[7]);
+                    acc[0] = f2_fma(v.x, ee.x, acc[0]);
+                    acc[1] = f2_fma(v.x, dd.x, acc[1]);
+                    acc[2] = f2_fma(v.x, em.y, acc[2]);
+                    acc[3] = f2_fma(v.x, dm.y, acc[3]);
+                    acc[4] = f2_fma(v.x, em.x, acc[4]);
+                    acc[5] = f2_fma(v.x, dm.x, acc[5]);
+                    acc[6] = f2_fma(v.x, eb.y, acc[6]);
+                    acc[7] = f2_fma(v.x, db.y, acc[7]);
+                    ee = em;
+                    em = eb;
+                    dd = dm;
+                    dm = db;
+                }
+            };
             // the lo products, summed by themselves
             float lo[kFilterOut];
             const int i0 = max(a0 - f.bl, 0), i1 = min(a0 + kFilterOut + f.bl, f.L4);
@@ -259,7 +292,10 @@ __global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const T* __
             // A high-pass sum is as large as its centre taps make it and small again once they are in, so the
             // bins next to the outputs, [a0 - 4, a0 + 12), are added one by one in row order (the centre
             // tap in its place) between the farther ones of either side: as few additions round at
-            // the large values as in a plain sum along the row (pairs throughout left 2.5 times its error).
+            // the large values as in a plain sum along the row (pairs throughout left 2.5 times its error).  The
+            // farther ones are added from either end towards the outputs, the small terms first; starting the
+            // right-hand ones with half of the sum so far in each half of a pair left that half to the end
+            // where a window's taps differ at even and odd offsets (cosine: twice a plain sum's error).
             const float* hi = tp + (f.c0 - a0);
             if (a0 > 4) conv(x, hi, hi + f.nt, a0 - 4);
             float v[kFilterOut];
@@ -298,14 +334,14 @@ __global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const T* __
             }
             const int right = a0 + 12;
 #pragma unroll
-            for (int o = 0; o < kFilterOut; ++o) acc[o] = f2_pack(0.5f * v[o], 0.5f * v[o]);
-            if (right < f.L4) conv(x + right, hi + right, hi + f.nt + right, f.L4 - right);
+            for (int o = 0; o < kFilterOut; ++o) acc[o] = 0ull;
+            if (right < f.L4) conv_back(x + right, hi + right, hi + f.nt + right, f.L4 - right);
 #pragma unroll
             for (int o = 0; o < kFilterOut; ++o) {
                 float p, q;
                 f2_unpack(acc[o], &p, &q);
                 const int a = a0 + o, dd = HALF ? 2 * a + s : a;
-                if (dd < D) res[dd] = (p + q) + lo[o];
+                if (dd < D) res[dd] = (v[o] + (p + q)) + lo[o];
             }
         }
     }
