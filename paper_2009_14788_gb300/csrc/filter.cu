@@ -192,13 +192,17 @@ __global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const T* __
         }
     }
     // rows: with HALF the odd bins first (the even outputs' sum), then the even bins
+    bool odd_values = false;   // infinities or NaN
     for (int r = 0; r < nrows; ++r) {
         const T* src = in + (row0 + r) * D;
         float* y = rowmem + (size_t)r * f.row_floats;
-        for (int d = threadIdx.x; d < S * f.L4; d += blockDim.x)
-            y[HALF ? ((d & 1) ? d >> 1 : f.L4 + (d >> 1)) : d] = d < D ? to_f32(src[d]) : 0.0f;
+        for (int d = threadIdx.x; d < S * f.L4; d += blockDim.x) {
+            const float v = d < D ? to_f32(src[d]) : 0.0f;
+            odd_values = odd_values || !(fabsf(v) < INFINITY);
+            y[HALF ? ((d & 1) ? d >> 1 : f.L4 + (d >> 1)) : d] = v;
+        }
     }
-    __syncthreads();
+    odd_values = __syncthreads_or(odd_values) != 0;
     const int r = (int)threadIdx.x / tpr, t0 = (int)threadIdx.x - r * tpr;
     if (r < nrows) {
         const float* y = rowmem + (size_t)r * f.row_floats;
@@ -331,6 +335,13 @@ __global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const T* __
                         if (HALF && j + w == o + 1) v[o] = fmaf(s == 0 ? 0.0f : own[o], centre.x, v[o]);
                         v[o] = fmaf(xi[w], t[j + w - o + 12], v[o]);
                     }
+            }
+            if (HALF && odd_values) {
+                // an infinity or NaN among the bins whose taps are left out still makes the output NaN
+                float z = 0.0f;
+                for (int i = 0; i < f.L4; ++i) z = fmaf(0.0f, y[(1 - s) * f.L4 + i], z);
+#pragma unroll
+                for (int o = 0; o < kFilterOut; ++o) lo[o] += z;
             }
             const int right = a0 + 12;
 #pragma unroll
