@@ -151,7 +151,8 @@ __host__ __device__ inline FilterPlan filter_plan(int D) {
     f.bl = HALF ? kFilterNear / 2 : kFilterNear;
     f.ntl = 2 * f.bl + 24;
     f.tap_floats = (HALF ? 2 : 1) * 2 * (f.nt + f.ntl);
-    f.row_floats = (HALF ? 2 : 1) * f.L4 + (D + 3) / 4 * 4;
+    // an odd number of float4s: the rows that a warp reads at once lie in different banks
+    f.row_floats = (((HALF ? 2 : 1) * f.L4 + D + 3) / 4 | 1) * 4;
     return f;
 }
 
@@ -161,7 +162,7 @@ __host__ __device__ inline FilterPlan filter_plan(int D) {
 // offsets: the reversed taps lie in shared memory twice, the second copy shifted by one, and both
 // windows slide in registers, one 16-byte load of each per four bins.  With Ram-Lak the zero taps are
 // left out.  512 views of 725 bins, FP32: 73 us with one bin per scalar FMA, both tap parts and the
-// zeros; 24 us so (30 us under the other windows; 500 views of 4000 bins 2078 -> 306 us).
+// zeros; 23 us so (29 us under the other windows; 500 views of 4000 bins 2078 -> 306 us).
 template <typename T, bool HALF>
 __global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const T* __restrict__ in, T* __restrict__ out,
                                                                      const float2* __restrict__ taps, int D,
@@ -193,14 +194,14 @@ __global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const T* __
     }
     // rows: with HALF the odd bins first (the even outputs' sum), then the even bins
     bool odd_values = false;   // infinities or NaN
-    for (int r = 0; r < nrows; ++r) {
-        const T* src = in + (row0 + r) * D;
-        float* y = rowmem + (size_t)r * f.row_floats;
-        for (int d = threadIdx.x; d < S * f.L4; d += blockDim.x) {
-            const float v = d < D ? to_f32(src[d]) : 0.0f;
-            odd_values = odd_values || !(fabsf(v) < INFINITY);
-            y[HALF ? ((d & 1) ? d >> 1 : f.L4 + (d >> 1)) : d] = v;
-        }
+    // (an element's row by a multiplication: at most 64 rows of fewer than 2^16 bins leave its rounding no say)
+    const int bins = S * f.L4;
+    const float per_bins = 1.0f / (float)bins, per_D = 1.0f / (float)D;
+    for (int e = threadIdx.x; e < nrows * bins; e += blockDim.x) {
+        const int r = (int)(((float)e + 0.5f) * per_bins), d = e - r * bins;
+        const float v = d < D ? to_f32(in[(row0 + r) * D + d]) : 0.0f;
+        odd_values = odd_values || !(fabsf(v) < INFINITY);
+        rowmem[r * f.row_floats + (HALF ? ((d & 1) ? d >> 1 : f.L4 + (d >> 1)) : d)] = v;
     }
     odd_values = __syncthreads_or(odd_values) != 0;
     const int r = (int)threadIdx.x / tpr, t0 = (int)threadIdx.x - r * tpr;
@@ -357,10 +358,9 @@ __global__ void __launch_bounds__(kFilterThreads) filter_rows_kernel(const T* __
         }
     }
     __syncthreads();
-    for (int q = 0; q < nrows; ++q) {
-        T* dst = out + (row0 + q) * D;
-        const float* res = rowmem + (size_t)q * f.row_floats + S * f.L4;
-        for (int d = threadIdx.x; d < D; d += blockDim.x) dst[d] = from_f32<T>(res[d]);
+    for (int e = threadIdx.x; e < nrows * D; e += blockDim.x) {
+        const int q = (int)(((float)e + 0.5f) * per_D);
+        out[row0 * D + e] = from_f32<T>(rowmem[q * f.row_floats + S * f.L4 + (e - q * D)]);
     }
 }
 
@@ -385,20 +385,27 @@ template <typename T, bool HALF>
 cudaError_t filter_launch(const void* in, void* out, const float2* taps, int D, long long rows, cudaStream_t s) {
     const FilterPlan f = filter_plan<HALF>(D);
     const int groups = (HALF ? 2 : 1) * f.A8 / kFilterOut;
-    const int tpr = std::min(kFilterThreads, (groups + 31) / 32 * 32);
-    // Rows per CTA share its taps: as many as one CTA's threads and half an SM's shared memory hold while
-    // every SM keeps about eight rows' worth of warps.
+    // Threads per row: one per group of outputs, in whole warps or a warp's half, quarter or eighth.
+    int tpr = std::min(kFilterThreads, (groups + 31) / 32 * 32);
+    while (tpr > 4 && tpr <= 32 && tpr / 2 >= groups) tpr /= 2;
+    // Rows per CTA share its taps: two, or as many as 128 threads serve, while three CTAs' worth is left for
+    // every SM and two CTAs fit it.
     int rpc = 1;
     if ((size_t)(f.tap_floats + f.row_floats) * sizeof(float) > 227 * 1024)
         return filter_launch_long<T>(in, out, taps, D, rows, s);
-    while (rpc < 4 && (rpc + 1) * tpr <= kFilterThreads && rows >= (long long)(rpc + 1) * 152 * 8 &&
+    while ((rpc + 1) * tpr <= (rpc == 1 ? kFilterThreads : 128) && rows >= (long long)(rpc + 1) * 152 * 3 &&
            (size_t)(f.tap_floats + (rpc + 1) * f.row_floats) * sizeof(float) <= 112 * 1024)
         ++rpc;
+    // Laying out the taps is most of a short launch: few CTAs take more threads for it (us, 128 rows and 8192 rows
+    // of 64 | 128 | 256 bins, Ram-Lak: a warp or more per row and no others 5.6, 18.3 | 8.0, 28.0 | 12.1,
+    // 46.2; so 3.8, 8.6 | 4.6, 21.9 | 6.2, 46.2; one bin per scalar FMA 3.1, 11.0 | 5.2, 35.2 | 6.3, 122).
+    const long long ctas = (rows + rpc - 1) / rpc;
+    const int threads = std::max((rpc * tpr + 31) / 32 * 32, ctas <= 2 * 152 ? 256 : ctas <= 8 * 152 ? 128 : 32);
     const size_t smem = (size_t)(f.tap_floats + rpc * f.row_floats) * sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(filter_rows_kernel<T, HALF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)std::max<size_t>(smem, 48 * 1024));
     if (e != cudaSuccess) return e;
-    filter_rows_kernel<T, HALF><<<(unsigned)((rows + rpc - 1) / rpc), rpc * tpr, smem, s>>>(
+    filter_rows_kernel<T, HALF><<<(unsigned)ctas, threads, smem, s>>>(
         (const T*)in, (T*)out, taps, D, rows, rpc, tpr);
     return cudaGetLastError();
 }
