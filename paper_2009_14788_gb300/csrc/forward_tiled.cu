@@ -146,10 +146,10 @@ namespace radon {
 
 namespace {
 
-template <typename T, int MODE, int NG, int LN>
+template <typename T, int MODE, int NG, int LN, bool ROWS>
 cudaError_t launch_packed_ng(const CUtensorMap& mr, const CUtensorMap& mc, const FwdTiledArgs& a, dim3 grid,
                              size_t smem, cudaStream_t s) {
-    auto kern = forward_packed_kernel<T, MODE, NG, LN>;
+    auto kern = forward_packed_kernel<T, MODE, NG, LN, ROWS>;
     static size_t attr_bytes = 0;
     if (smem > attr_bytes) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -162,12 +162,16 @@ cudaError_t launch_packed_ng(const CUtensorMap& mr, const CUtensorMap& mc, const
 
 template <typename T, int MODE>
 cudaError_t launch_packed_t(const CUtensorMap& mr, const CUtensorMap& mc, const FwdTiledArgs& a, dim3 grid,
-                            size_t smem, int NG, int LN, cudaStream_t s) {
-    if (LN == 2) return launch_packed_ng<T, MODE, 1, 2>(mr, mc, a, grid, smem, s);
-    if constexpr (MODE == kMathScalar)
-        if (NG == 4) return launch_packed_ng<T, MODE, 4, 1>(mr, mc, a, grid, smem, s);
-    return NG == 2 ? launch_packed_ng<T, MODE, 2, 1>(mr, mc, a, grid, smem, s)
-                   : launch_packed_ng<T, MODE, 1, 1>(mr, mc, a, grid, smem, s);
+                            size_t smem, int NG, int LN, bool rows, cudaStream_t s) {
+    if (LN == 2) return launch_packed_ng<T, MODE, 1, 2, false>(mr, mc, a, grid, smem, s);
+    if constexpr (MODE == kMathScalar) {
+        if (NG == 4) return launch_packed_ng<T, MODE, 4, 1, true>(mr, mc, a, grid, smem, s);
+        if (rows)
+            return NG == 2 ? launch_packed_ng<T, MODE, 2, 1, true>(mr, mc, a, grid, smem, s)
+                           : launch_packed_ng<T, MODE, 1, 1, true>(mr, mc, a, grid, smem, s);
+    }
+    return NG == 2 ? launch_packed_ng<T, MODE, 2, 1, false>(mr, mc, a, grid, smem, s)
+                   : launch_packed_ng<T, MODE, 1, 1, false>(mr, mc, a, grid, smem, s);
 }
 
 }  // namespace
@@ -277,27 +281,15 @@ radon_status launch_forward_packed(radon_geometry* g, const void* packed, void* 
     const radon_status st =
         packed_forward_shape(g, dt, batch, cfg, dt == RADON_F16 && fp16_weights(cfg, ep), lanes, &sh, why);
     if (st != RADON_OK) return st;
-    const int G = sh.G, Dt = sh.Dt, NG = sh.NG, LN = sh.LN, R = sh.R, wbox = sh.wbox, stages = sh.stages;
-    const size_t smem = sh.smem;
+    const int G = sh.G, Dt = sh.Dt, LN = sh.LN, R = sh.R, wbox = sh.wbox;
     int gi = 0;
     while ((1 << gi) < G) ++gi;
     const int groups = (batch + BG - 1) / BG;
     const uint64_t n = (uint64_t)g->n;
     const uint64_t dims[4] = {(uint64_t)BG, n, n, (uint64_t)groups};
     const uint64_t strides[3] = {16, n * 16, n * n * 16};
-    const uint32_t box[4] = {(uint32_t)BG, (uint32_t)wbox, (uint32_t)(R + 2), (uint32_t)NG};
     const unsigned char* rows = reinterpret_cast<const unsigned char*>(packed);
     const unsigned char* cols = rows + (size_t)groups * n * n * 16;
-    CUtensorMap mr, mc;
-    int rc = encode_tiled(&mr, tma_dtype(dt), 4, const_cast<unsigned char*>(rows), dims, strides, box,
-                          CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
-    if (rc == 0)
-        rc = encode_tiled(&mc, tma_dtype(dt), 4, const_cast<unsigned char*>(cols), dims, strides, box,
-                          CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
-    if (rc != 0) {
-        *why = "cuTensorMapEncodeTiled rejected the packed-image descriptor (CUresult " + std::to_string(rc) + ")";
-        return RADON_ERR_UNSUPPORTED;
-    }
     FwdTiledArgs a;
     a.rays = g->d_ray;
     a.nks = g->d_nk;
@@ -326,24 +318,57 @@ radon_status launch_forward_packed(radon_geometry* g, const void* packed, void* 
         return RADON_ERR_CUDA;
     }
     a.spin_limit = kSpinLimit;
-    a.stages = stages;
     a.vec_store = (g->D % 2 == 0 && ((uintptr_t)sino % (2 * esz)) == 0) ? 1 : 0;
     const long long nblk = (long long)g->group_count[gi] * a.n_dr;
-    dim3 grid((unsigned)nblk, (unsigned)((groups + NG - 1) / NG));
-    cudaError_t e;
-    switch (dt) {
-        case RADON_F16:
-            e = fp16_weights(cfg, ep) ? launch_packed_t<__half, kMathF16W>(mr, mc, a, grid, smem, NG, LN, s)
-                                      : launch_packed_t<__half, kMathScalar>(mr, mc, a, grid, smem, NG, LN, s);
-            break;
-        case RADON_BF16: e = launch_packed_t<__nv_bfloat16, kMathScalar>(mr, mc, a, grid, smem, NG, LN, s); break;
-        default: e = launch_packed_t<float, kMathScalar>(mr, mc, a, grid, smem, NG, LN, s); break;
+    const bool f16w = dt == RADON_F16 && fp16_weights(cfg, ep);
+    // Groups [g0, g0 + count) in CTAs of NG groups.
+    auto launch = [&](int g0, int count, int NG, int stages, size_t smem, bool by_rows) {
+        const uint32_t box[4] = {(uint32_t)BG, (uint32_t)wbox, (uint32_t)(R + 2), (uint32_t)NG};
+        CUtensorMap mr, mc;
+        int rc = encode_tiled(&mr, tma_dtype(dt), 4, const_cast<unsigned char*>(rows), dims, strides, box,
+                              CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
+        if (rc == 0)
+            rc = encode_tiled(&mc, tma_dtype(dt), 4, const_cast<unsigned char*>(cols), dims, strides, box,
+                              CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
+        if (rc != 0) {
+            *why = "cuTensorMapEncodeTiled rejected the packed-image descriptor (CUresult " + std::to_string(rc) + ")";
+            return RADON_ERR_UNSUPPORTED;
+        }
+        a.g0 = g0;
+        a.stages = stages;
+        const dim3 grid((unsigned)nblk, (unsigned)((count + NG - 1) / NG));
+        cudaError_t e;
+        switch (dt) {
+            case RADON_F16:
+                e = f16w ? launch_packed_t<__half, kMathF16W>(mr, mc, a, grid, smem, NG, LN, by_rows, s)
+                         : launch_packed_t<__half, kMathScalar>(mr, mc, a, grid, smem, NG, LN, by_rows, s);
+                break;
+            case RADON_BF16:
+                e = launch_packed_t<__nv_bfloat16, kMathScalar>(mr, mc, a, grid, smem, NG, LN, by_rows, s);
+                break;
+            default: e = launch_packed_t<float, kMathScalar>(mr, mc, a, grid, smem, NG, LN, by_rows, s); break;
+        }
+        if (e != cudaSuccess) {
+            *why = std::string("packed forward launch: ") + cudaGetErrorString(e);
+            return RADON_ERR_CUDA;
+        }
+        return RADON_OK;
+    };
+    // One or two groups past whole CTAs of four run by themselves, row by row like the others with the same slabs, so
+    // that equal images of a batch have equal projections; and with their code out of the kernel of four
+    // groups it keeps its registers (us, one launch that takes them sample by sample -> two: 32 x 512^2, 512
+    // views, no tail, FP16 1387 -> 1352, BF16 1283 -> 1206; 34 FP16 images 1988 -> 1941, 41 2182 -> 2187; FP32 38
+    // x 256^2, 256 views 339 -> 324).  Two groups take two CTAs per SM (96 registers; at three 72 spill: 41 2220).
+    const int tail = sh.NG == 4 && groups % 4 <= 2 ? groups % 4 : 0;
+    radon_status done = launch(0, groups - tail, sh.NG, sh.stages, sh.smem, sh.NG == 4);
+    if (done == RADON_OK && tail > 0) {
+        int stages = 2;
+        while (stages < kFwdMaxStages && fwd_packed_smem_bytes(R, wbox, stages + 1, tail) <= (tail == 2 ? 113 : 75) * 1024) ++stages;
+        done = launch(groups - tail, tail, tail, stages, fwd_packed_smem_bytes(R, wbox, stages, tail), true);
+        if (done == RADON_OK) count_launches(1);
+        else if (done == RADON_ERR_UNSUPPORTED) done = RADON_ERR_CUDA;   // the first launch has run: no other path
     }
-    if (e != cudaSuccess) {
-        *why = std::string("packed forward launch: ") + cudaGetErrorString(e);
-        return RADON_ERR_CUDA;
-    }
-    return RADON_OK;
+    return done;
 }
 
 }  // namespace radon

@@ -63,6 +63,7 @@ struct FwdTiledArgs {
     Epilogue ep;
     int stages;           // compute buffers in the ring (packed: 2..4; repacking: 2)
     int vec_store;        // 1: D even and the sinogram aligned to two elements (paired stores)
+    int g0;               // packed: the launch's first texel group
 };
 
 // Two consecutive outputs as one 4-byte (16-bit storage) or 8-byte (FP32) store; `p` is aligned to
@@ -401,7 +402,7 @@ struct FwdRow {
 // ray (rays where bands of 256 detectors per view would not fit a TMA box): lane `sub` takes the
 // ray's samples sub, sub + 2, ... of every slab, the two lanes agree on where the slab's samples end,
 // and their partial sums meet in one shuffle before the store.
-template <typename T, int MODE, int NG = 1, int LN = 1>
+template <typename T, int MODE, int NG = 1, int LN = 1, bool ROWS = false>
 __device__ void fwd_consume(const FwdTiledArgs& a, int cls, int v0, int cnt, int d0, int b0, uint64_t* full,
                             uint64_t* empty, const int* band_xc0, const int* band_bad, volatile int* abort_flag,
                             const unsigned char* comp_base, size_t comp_stride, int wc, int* slab_rng,
@@ -441,12 +442,12 @@ __device__ void fwd_consume(const FwdTiledArgs& a, int cls, int v0, int cnt, int
         }
     }
     const float dX = dXh + dXl, dY = dYh + dYl;
-    // Four texel groups go row by row (see FwdRow) where at most three of the ray's samples reach a texel
-    // row, over at most four columns: steps of one pixel within 48 degrees of the rows' normal, i.e. every
-    // parallel ray and all but the steepest of a fan.  Other rays, and CTAs of one or two groups, over
-    // which a row's weights do not pay (8 BF16 images 126 -> 151 us, 16 FP16 images 1.39 -> 1.38 ms), go
-    // sample by sample.
-    const bool by_row = NG == 4 && nk > 0 && dY >= kRowMinStep && dY <= 1.0001f && fabsf(dX) <= 0.75f;
+    // Launches of four texel groups per CTA go row by row (see FwdRow) where at most three of the ray's samples
+    // reach a texel row, over at most four columns: every parallel ray with steps of one pixel and all but
+    // the steepest of such a fan; with shorter steps the rays nearest the rows' normal, down to 0.668 rows a
+    // step.  Other rays, and launches of one or two groups, over which a row's weights do not pay (8 BF16
+    // images 126 -> 151 us, 16 FP16 images 1.39 -> 1.38 ms), go sample by sample.
+    const bool by_row = ROWS && nk > 0 && dY >= kRowMinStep && dY <= 1.0001f && fabsf(dX) <= 0.75f;
     const float rdY = by_row ? 1.0f / dY : 0.0f;
     int r_lo = 0, r_hi = -1;   // texel rows the ray's samples reach
     if (by_row) {
@@ -749,8 +750,9 @@ __global__ void __launch_bounds__(kFwdThreads, 3) forward_tiled_kernel(const __g
 // Packed variant: the image batch was packed once into 16-byte texels (rows / cols copies, see
 // pack.cu), so the producer warp only bounds each band and copies it with one 4-D TMA load straight
 // into the compute buffer it will become (row pitch = band width); no staging, no repack.
-template <typename T, int MODE, int NG, int LN>
-__global__ void __launch_bounds__(kFwdThreads, NG == 4 ? 2 : 3) forward_packed_kernel(const __grid_constant__ CUtensorMap map_rows,
+// ROWS: rays go row by row where they can (four groups, and the one or two left over from a launch of four).
+template <typename T, int MODE, int NG, int LN, bool ROWS>
+__global__ void __launch_bounds__(kFwdThreads, ROWS && NG >= 2 ? 2 : 3) forward_packed_kernel(const __grid_constant__ CUtensorMap map_rows,
                                                                        const __grid_constant__ CUtensorMap map_cols,
                                                                        const FwdTiledArgs a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -775,7 +777,7 @@ __global__ void __launch_bounds__(kFwdThreads, NG == 4 ? 2 : 3) forward_packed_k
     const Int2 grp = a.groups[grp_idx];
     const int v0 = grp.x, cnt = grp.y & 0xffff, cls = grp.y >> 16;
     const int d0 = dr * a.Dt;
-    const int b0 = blockIdx.y * NG * Texel<T>::BG;
+    const int g0 = a.g0 + blockIdx.y * NG, b0 = g0 * Texel<T>::BG;
 
     if (tid < a.stages) {
         mbar_init(&full[tid], 1);
@@ -815,7 +817,7 @@ __global__ void __launch_bounds__(kFwdThreads, NG == 4 ? 2 : 3) forward_packed_k
                     // NG groups' planes in one box (a group past the batch's last reads as zeros)
                     mbar_arrive_expect_tx(&full[buf], (uint32_t)NG * plane);
                     tma_load_4d(comp_base + (size_t)buf * comp_stride, map, &full[buf], 0, band.xc0, -4 + s * a.R,
-                                (int)blockIdx.y * NG);
+                                g0);
                 }
             }
             __syncwarp();
@@ -823,16 +825,12 @@ __global__ void __launch_bounds__(kFwdThreads, NG == 4 ? 2 : 3) forward_packed_k
         }
         return;
     }
-    const int left = a.B - b0;   // images from here on: groups past the batch read as zeros or not at all
-    if (NG == 4 && left > 2 * Texel<T>::BG)
-        fwd_consume<T, MODE, NG, LN>(a, cls, v0, cnt, d0, b0, full, empty, band_xc0, band_bad, abort_flag,
-                                     comp_base, comp_stride, a.wbox, slab_rng, plane);
-    else if (NG >= 2 && left > Texel<T>::BG)
-        fwd_consume<T, MODE, NG >= 2 ? 2 : 1, LN>(a, cls, v0, cnt, d0, b0, full, empty, band_xc0, band_bad, abort_flag,
-                                                  comp_base, comp_stride, a.wbox, slab_rng, plane);
-    else
-        fwd_consume<T, MODE, 1, LN>(a, cls, v0, cnt, d0, b0, full, empty, band_xc0, band_bad, abort_flag,
-                                    comp_base, comp_stride, a.wbox, slab_rng);
+    if (NG == 4 || (NG == 2 && b0 + Texel<T>::BG < a.B))
+        fwd_consume<T, MODE, NG, LN, ROWS>(a, cls, v0, cnt, d0, b0, full, empty, band_xc0, band_bad, abort_flag,
+                                           comp_base, comp_stride, a.wbox, slab_rng, plane);
+    else   // one group (or a pair whose second group lies past the batch: its plane is never read)
+        fwd_consume<T, MODE, 1, LN, ROWS>(a, cls, v0, cnt, d0, b0, full, empty, band_xc0, band_bad, abort_flag,
+                                          comp_base, comp_stride, a.wbox, slab_rng);
 }
 
 }  // namespace radon
