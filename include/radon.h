@@ -322,14 +322,15 @@ RADON_API radon_status radon_forward_static_scratch(const radon_geometry* geomet
  * 8- or 16-image groups reads the weights instead of evaluating them: the same nonzero products added
  * in the same order, so the same bits.  A parallel beam's weights are cheaper to evaluate than to read
  * (all rays of a view share one step): there only groups of 16 images with a sampling step of
- * sqrt(2) * 2 / 3 or less read the table.
- *   - radon_geometry_adjoint_table_size: the table's device bytes, tiles x views x (128 pairs x 44
- *     + 4) (4.2 GB for 512^2 and 720 views); no allocation.
+ * sqrt(2) * 2 / 3 or less read the table, and with longer steps none is built.
+ *   - radon_geometry_adjoint_table_size: the device bytes of a table, tiles x views x (128 pairs x 44
+ *     + 4) (4.2 GB for 512^2 and 720 views), whether or not one is built; no allocation.
  *   - radon_geometry_build_adjoint_table: allocates the table on the geometry's device (which must be
  *     current) and fills it; synchronises the device; not capturable.  RADON_ERR_UNSUPPORTED (nothing
  *     kept) where the packed adjoint cannot serve the geometry (a detector window wider than 256 or a
  *     sampling step of sqrt(2) / 3 or less), RADON_ERR_OOM when the device memory runs out.  Building
- *     again replaces the table.
+ *     again replaces the table.  For a parallel beam with a step above sqrt(2) * 2 / 3, where no call would
+ *     read it, RADON_OK with nothing allocated, launched or kept.
  *   - radon_geometry_adjoint_table_overflow: the fraction of (pair, view) records left to the
  *     on-the-fly weights (0 without a table).
  *   - radon_geometry_free_adjoint_table: frees it (radon_geometry_destroy does too); the adjoint then

@@ -144,6 +144,7 @@ radon_status build_adjoint_table(radon_geometry* g, std::string* why) {
         return RADON_ERR_UNSUPPORTED;
     }
     free_adjoint_table(g);
+    if (!g->fan && kw == 3) return RADON_OK;   // no group reads it (bwdp_table_serves): nothing to build or keep
     const int tiles_x = (g->n + kBwdTile - 1) / kBwdTile;
     const size_t recs = (size_t)tiles_x * tiles_x * (size_t)g->V * kBwdTabPairs;
     float4* w = nullptr;
@@ -169,8 +170,7 @@ radon_status build_adjoint_table(radon_geometry* g, std::string* why) {
     if (e == cudaSuccess) e = cudaMemset(vflag, 0, tv * sizeof(int));
     if (e == cudaSuccess) {
         const dim3 grid((unsigned)(tiles_x * tiles_x), (unsigned)((g->V + kViewsPerBlock - 1) / kViewsPerBlock));
-        auto kern = g->fan ? (kw == 3 ? bwdp_table_kernel<3, false> : bwdp_table_kernel<6, false>)
-                           : (kw == 3 ? bwdp_table_kernel<3, true> : bwdp_table_kernel<6, true>);
+        auto kern = !g->fan ? bwdp_table_kernel<6, true> : kw == 3 ? bwdp_table_kernel<3, false> : bwdp_table_kernel<6, false>;
         kern<<<grid, kBwdTabPairs>>>(g->d_ray, g->d_view, g->n, g->V, g->D, bwdp_lattice(g), wd, tiles_x, kViewsPerBlock, w, w5, la,
                                      vflag, over);
         e = cudaGetLastError();

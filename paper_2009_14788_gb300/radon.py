@@ -113,16 +113,18 @@ class Geometry:
         return rays, counts
 
     def adjoint_table_bytes(self) -> int:
-        """Device bytes of the exact adjoint's weight table (see ``build_adjoint_table``)."""
+        """Device bytes of the exact adjoint's weight table, built or not (see ``build_adjoint_table``)."""
         b = ctypes.c_size_t()
         L.check(L.radon_geometry_adjoint_table_size(self._h, ctypes.byref(b)), "radon_geometry_adjoint_table_size")
         return int(b.value)
 
     def build_adjoint_table(self) -> None:
         """Precomputes the exact adjoint's bilinear weights on the geometry's device (tiles x views x 128
-        pixel pairs x 44 bytes, ``adjoint_table_bytes``); the packed adjoint then reads them instead of
-        computing them, with the same bits (pixel pairs whose weighted rays span more than five detectors
-        in a view keep computing theirs: ``adjoint_table_overflow``).  Raises ``RadonError``
+        pixel pairs x 44 bytes, ``adjoint_table_bytes``); the packed adjoint of a fan beam then reads them
+        instead of computing them in groups of 8 and 16 images, with the same bits (pixel pairs whose weighted
+        rays span more than five detectors in a view keep computing theirs: ``adjoint_table_overflow``).  A
+        parallel beam's weights are cheaper to compute: only groups of 16 images with a step of sqrt(2) * 2 / 3
+        or less read them, and with longer steps this call does nothing.  Raises ``RadonError``
         (RADON_ERR_UNSUPPORTED) where the packed adjoint cannot serve the geometry."""
         with torch.cuda.device(self.device):
             L.check(L.radon_geometry_build_adjoint_table(self._h), "radon_geometry_build_adjoint_table")
@@ -599,8 +601,8 @@ class Radon:
     backward = backprojection
 
     def build_adjoint_table(self) -> None:
-        """Precomputes the exact adjoint's weights for this geometry (``Geometry.build_adjoint_table``):
-        batched backprojections then read them, with the same bits."""
+        """Precomputes the exact adjoint's weights for this geometry where batched backprojections read them
+        (fan beams, and parallel beams of short steps: ``Geometry.build_adjoint_table``), with the same bits."""
         self.geometry.build_adjoint_table()
 
     def filter_sinogram(self, sino: torch.Tensor, filter_name: str = "ram-lak") -> torch.Tensor:
