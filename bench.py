@@ -182,12 +182,15 @@ def roofline(samples, ms, sm_count, per_sm, clk_mhz, basis, traffic):
 # ----------------------------------------------------------------------------- GPU arm
 
 def _try_adjoint_table(geom, L):
-    """Builds the geometry's adjoint weight table (once per geometry, outside any timed region);
-    returns (bytes, seconds, overflow fraction) or None where the library refuses it."""
-    t0 = time.perf_counter()
+    """Builds the geometry's adjoint weight table (once per geometry, outside any timed region); returns
+    (bytes, seconds, overflow fraction) or None where the library refuses it or, for parallel beams of
+    longer steps, keeps none."""
+    t0, launched = time.perf_counter(), L.radon_kernel_launch_count()
     try:
         geom.build_adjoint_table()
     except L.RadonError:
+        return None
+    if L.radon_kernel_launch_count() == launched:
         return None
     return geom.adjoint_table_bytes(), time.perf_counter() - t0, geom.adjoint_table_overflow()
 
@@ -549,17 +552,15 @@ def run_secondary(args):
 
     * Landweber (8 x 512^2 parallel, 60 views in [0, pi), 725 detectors, bf16 storage): the step
       size by 20 power iterations, 10 Landweber iterations forward, and the reverse pass to the
-      gradients w.r.t. y and alpha (per-iteration checkpoints: 3 projections per iteration); the
-      iterations again with the geometry's adjoint weight table.
+      gradients w.r.t. y and alpha (per-iteration checkpoints: 3 projections per iteration, less the last
+      adjoint, which only a gradient w.r.t. x_0 needs).
     * The paper's batch benchmark shape (32 x 512^2 parallel, 512 views in [0, pi), 512
-      detectors): forward + adjoint, chosen 16-bit form against the plain FP32 form, without and
-      with the geometry's adjoint weight table.
+      detectors): forward + adjoint, chosen 16-bit form against the plain FP32 form.
     * The uneven batch (64 images, 16 each of 128^2 .. 1024^2, each with its own parallel geometry,
       fp16): one forward plan and one adjoint plan (autotuned at creation) replayed as one CUDA
       graph, against one library call per image and direction.
     * Filtered backprojection at the paper's FBP setting (512^2, 512 views, 725 detectors, Ram-Lak),
-      and CGNE (20 iterations) at the same setting; the batched ones also with the geometry's adjoint
-      weight table.
+      and CGNE (20 iterations) at the same setting.
     * The pixel-driven interpolating backprojector against the exact adjoint on the headline workload.
     """
     import torch
@@ -613,14 +614,8 @@ def run_secondary(args):
         loss = ((xk.float() - xt) ** 2).sum()
         loss.backward()
     ms_fb = time_it(fwd_bwd, 3)
-    # the same with the geometry's adjoint weight table (its 8-image groups read the weights)
-    tab = _try_adjoint_table(g, L)
-    ms_fwd_t = time_it(lambda: lw.run(x0, yg, ag, K), 3) if tab is not None else None
-    ms_fb_t = time_it(fwd_bwd, 3) if tab is not None else None
-    if tab is not None:
-        g.free_adjoint_table()
     proj_fwd = 2 * K * w.batch * S
-    proj_bwd = 3 * K * w.batch * S
+    proj_bwd = (3 * K - 1) * w.batch * S   # no gradient to x_0: the last adjoint is left out
     out["landweber"] = {
         "workload": w.name, "storage": "bf16", "iterations": K, "power_iterations": P,
         "lambda": float(lam.item()), "alpha": float(alpha.item()),
@@ -628,9 +623,6 @@ def run_secondary(args):
         "samples_per_s_forward": proj_fwd / (ms_fwd * 1e-3),
         "samples_per_s_forward_backward": (proj_fwd + proj_bwd) / (ms_fb * 1e-3),
         "samples_per_s_power_iteration": 2 * P * S / (ms_power * 1e-3),
-        "with_adjoint_table": (None if tab is None else
-                               {"bytes": tab[0], "ms_forward": ms_fwd_t, "ms_forward_backward": ms_fb_t,
-                                "samples_per_s_forward_backward": (proj_fwd + proj_bwd) / (ms_fb_t * 1e-3)}),
         "l2": "flushed (2x L2 write) before each timed iteration",
     }
     del g, xt, y32, y, yg, ag, x0
@@ -657,25 +649,6 @@ def run_secondary(args):
         del x, yb, oy, ox
     res["speedup_chosen_vs_plain_f32"] = res["plain_f32"]["ms_per_step"] / res["chosen_f16"]["ms_per_step"]
     res["speedup_chosen_vs_tuned_f32"] = res["tuned_f32"]["ms_per_step"] / res["chosen_f16"]["ms_per_step"]
-    # the same two tuned forms with the geometry's adjoint weight table (16-image groups reading it)
-    tab = _try_adjoint_table(g, L)
-    if tab is not None:
-        res["adjoint_table_bytes"] = tab[0]
-        for label, dt in (("chosen_f16_table", torch.float16), ("tuned_f32_table", torch.float32)):
-            cfg = launch_config("auto")
-            x = torch.from_numpy(xs).to("cuda", dt)
-            yb = forward_raw(g, x, cfg)
-            oy, ox = torch.empty_like(yb), torch.empty_like(x)
-
-            def fa():
-                forward_raw(g, x, cfg, out=oy)
-                backward_raw(g, yb, cfg, out=ox)
-            ms = time_it(fa, 5, warm=1)
-            res[label] = {"ms_per_step": ms, "samples_per_s": 2 * B * S / (ms * 1e-3), "images_per_s": B / (ms * 1e-3)}
-            del x, yb, oy, ox
-        g.free_adjoint_table()
-        res["speedup_chosen_table_vs_plain_f32"] = (res["plain_f32"]["ms_per_step"] /
-                                                    res["chosen_f16_table"]["ms_per_step"])
     out["paper_batch"] = res
     del xs
     # the uneven batch: 64 images of 128^2..1024^2, each with its own geometry, in one persistent
@@ -758,9 +731,7 @@ def run_secondary(args):
     g = Geometry("parallel", 512, uniform_angles(512, np.pi), det_count=D, det_spacing=1.0)
     res = {"workload": "parallel_n512_v512_d725_ramlak", "storage": "f32",
            "l2": "flushed (2x L2 write) before each timed call"}
-    for B, table in ((1, False), (16, False), (16, True)):
-        if table and _try_adjoint_table(g, L) is None:
-            continue
+    for B in (1, 16):
         x = torch.from_numpy(np.stack([ellipse_phantom(512, 10, 4242 + b) for b in range(B)])).to("cuda", torch.float32)
         y = forward_raw(g, x)
         q = torch.empty_like(y)
@@ -771,26 +742,21 @@ def run_secondary(args):
             filter_sinogram(g, y, "ram-lak", out=q)
             backward_raw(g, q, out=rec)
         ms_fbp = time_it(fbp, 5)
-        res["batch%d%s" % (B, "_table" if table else "")] = {"ms_filter": ms_f, "ms_fbp": ms_fbp,
-                                                            "images_per_s": B / (ms_fbp * 1e-3)}
+        res["batch%d" % B] = {"ms_filter": ms_f, "ms_fbp": ms_fbp, "images_per_s": B / (ms_fbp * 1e-3)}
         del x, y, q, rec
-    g.free_adjoint_table()
     out["fbp"] = res
     # CGNE at the same setting (Section 4.2 runs 500 iterations): 20 iterations, batch 1 and 8
     from paper_2009_14788_gb300 import cgne
     res = {"workload": "parallel_n512_v512_d725", "storage": "f32", "iterations": 20,
            "l2": "flushed (2x L2 write) before each timed call"}
-    for B, table in ((1, False), (8, False), (8, True)):
-        if table and _try_adjoint_table(g, L) is None:
-            continue
+    for B in (1, 8):
         x = torch.from_numpy(np.stack([ellipse_phantom(512, 10, 4242 + b) for b in range(B)])).to("cuda", torch.float32)
         y = forward_raw(g, x)
         x0 = torch.zeros_like(x)
         ms = time_it(lambda: cgne(g, x0, y, 20), 3, warm=1)
-        res["batch%d%s" % (B, "_table" if table else "")] = {
+        res["batch%d" % B] = {
             "ms": ms, "ms_per_iteration": ms / 20, "samples_per_s": 2 * 20 * B * g.sample_count / (ms * 1e-3)}
         del x, y, x0
-    g.free_adjoint_table()
     out["cgne"] = res
     # the pixel-driven interpolating backprojector against the exact adjoint, headline workload
     from paper_2009_14788_gb300 import backproject_interpolating
