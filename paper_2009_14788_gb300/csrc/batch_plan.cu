@@ -153,9 +153,12 @@ constexpr int kPlanMaxLanes = 4;
 // 32 samples.  Bound by issue and by the FMA pipe about alike, so four samples per loop turn share its
 // bookkeeping and have their loads in flight together, and the two texel rows keep sums of their own
 // (joined at the end).  Pairing the arithmetic as f32x2 took a third of the instructions away but no time:
-// a pair costs the FMA pipe two cycles and half a cycle more next to scalar instructions.  Six CTAs per SM
-// (40 registers) cover the loads' latency better than five: 1.92 -> 1.75 ms for eight FP16 images of
-// 128^2 .. 1024^2 (1.97 with one sample per loop turn).
+// a pair costs the FMA pipe two cycles and half a cycle more next to scalar instructions.  Four CTAs per SM (64
+// registers, of which the four samples' positions and texels take their share) beat six of 40, which had to
+// order the loads and, in FP32, to spill (us, one sample per loop turn -> 40 registers -> 64: eight images of
+// 128^2 .. 1024^2 FP16 1966 -> 1757 -> 1754, BF16 1943 -> 1759 -> 1601, FP32 1994 -> 1844 -> 1764; one image
+// with its packing, FP32, 512^2 and 512 views 203 -> 188 -> 162, 128^2 and 180 views 15.4 -> 16.4 -> 11.5, 64^2
+// and 64 views 10.0 -> 10.9 -> 7.8).
 template <typename T, int LANES>
 __device__ float plan_ray(const Unit& u, const typename Quad<T>::type* __restrict__ quads, int v, int d, int sub) {
     const long long r = (long long)v * u.D + d;
@@ -280,7 +283,7 @@ __device__ __forceinline__ int next_work(bool first, unsigned* counter) {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kPlanThreads, 6) plan_forward_kernel(const Unit* __restrict__ units,
+__global__ void __launch_bounds__(kPlanThreads, 4) plan_forward_kernel(const Unit* __restrict__ units,
                                                                     const Work* __restrict__ work, int n_work,
                                                                     unsigned* counter,
                                                                     const typename Quad<T>::type* __restrict__ quads) {
@@ -298,7 +301,7 @@ __global__ void __launch_bounds__(kPlanThreads, 6) plan_forward_kernel(const Uni
 
 // Single image (a batch-1 call): the same work items, one CTA each, the unit passed by value.
 template <typename T>
-__global__ void __launch_bounds__(kPlanThreads, 6) single_forward_kernel(const Unit u,
+__global__ void __launch_bounds__(kPlanThreads, 4) single_forward_kernel(const Unit u,
                                                                       const typename Quad<T>::type* __restrict__ quads,
                                                                       const Epilogue ep) {
     plan_forward_tile<T>(u, (int)blockIdx.x, quads, ep);
