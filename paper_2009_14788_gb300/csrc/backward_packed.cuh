@@ -190,7 +190,9 @@ struct BwdPPar {
 
 __device__ __forceinline__ BwdPPar bwdp_par_view(const ViewF vf, const RayT* __restrict__ rays, int v, int D, int n,
                                                  int dlo, int ti, int tj, const BwdPLattice g) {
-    const BwdTileRay A = bwd_tile_ray(vf, rays + (long long)v * D, D, n, ti, tj, g.ih2, g.nh, g.nl);
+    const float cx = 0.5f * (float)min(kBwdTile - 1, n - 1 - tj), cy = 0.5f * (float)min(kBwdTile - 1, n - 1 - ti);
+    const BwdTileRay A = bwd_tile_ray(vf, rays + (long long)v * D, D, bwd_det_affine(vf, (float)tj + cx, (float)ti + cy), ti,
+                                      tj, g.ih2, g.nh, g.nl);
     const float bx = A.sx * g.ih2, by = A.sy * g.ih2;
     BwdPPar w;
     w.nx = A.nx;

@@ -178,12 +178,11 @@ struct BwdTileRay {
     int d;
 };
 
-__device__ __forceinline__ BwdTileRay bwd_tile_ray(const ViewF& vf, const RayT* __restrict__ rays, int D, int n, int ti,
+// `t`: the detector coordinate of the centre of the tile's pixels; `rays`: the view's.
+__device__ __forceinline__ BwdTileRay bwd_tile_ray(const ViewF& vf, const RayT* __restrict__ rays, int D, float t, int ti,
                                                    int tj, float ih2, float nh, float nl) {
-    const float cx = 0.5f * (float)min(kBwdTile - 1, n - 1 - tj), cy = 0.5f * (float)min(kBwdTile - 1, n - 1 - ti);
-    const float t = rintf(bwd_det_affine(vf, (float)tj + cx, (float)ti + cy));
     BwdTileRay w;
-    w.d = (int)fminf(fmaxf(t, 0.0f), (float)(D - 1));
+    w.d = (int)fminf(fmaxf(rintf(t), 0.0f), (float)(D - 1));
     const RayT ray = rays[w.d];
     w.sx = ray.dxh + ray.dxl;
     w.sy = ray.dyh + ray.dyl;

@@ -27,6 +27,7 @@
 #include <map>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "backward_tiled.cuh"
@@ -483,22 +484,26 @@ __device__ void plan_adjoint_tile_parallel(const Unit& u, int tile, const AdjBuf
     const int wp = NC > 0 ? wd + kAdjPad : wd;   // staged values per view
     const float inv_wp = 1.0f / (float)wp, wd_last = (float)(wd - 1);
     const uint32_t ys_a = smem_u32(b.ys), par_a = smem_u32(b.sh->par);
+    const float ih2 = u.ih2, nh = u.nh, nl = u.nl;   // (loaded once: a plan's unit lies in global memory)
     float acc0 = 0.0f, acc1 = 0.0f;
     for (int c0 = 0; c0 < u.V; c0 += CV) {
         const int nv = min(CV, u.V - c0);
         if (tid < nv) {
             const ViewF vf = u.views[c0 + tid];
-            int dlo;
-            float r;
-            bwd_view_window(vf, ti, tj, u.n, &dlo, &r);
-            // every pixel's candidates [ceil(t - r), floor(t + r)] within the detector must lie in the
-            // staged window (the tile's largest t is at a corner); a miss is recorded, not overrun
+            // the tile's window as bwd_view_window gives it, without that function's divisions (the map's
+            // denominator is one): the other warps wait for this one in every chunk (one image of 224^2 and
+            // 492 views 101 -> 98 us)
             const float x1 = (float)(tj + xe), y1 = (float)(ti + ye);
             const float t00 = bwd_det_affine(vf, (float)tj, (float)ti), t10 = bwd_det_affine(vf, x1, (float)ti);
             const float t01 = bwd_det_affine(vf, (float)tj, y1), t11 = bwd_det_affine(vf, x1, y1);
             const float tmax = fmaxf(fmaxf(t00, t10), fmaxf(t01, t11)), tmin = fminf(fminf(t00, t10), fminf(t01, t11));
+            const float r = fabsf(vf.ax) + fabsf(vf.ay) + 0.01f;
+            const int dlo = (int)floorf(tmin - r - 0.01f);
+            // every pixel's candidates [ceil(t - r), floor(t + r)] within the detector must lie in the
+            // staged window (the tile's largest t is at a corner); a miss is recorded, not overrun
             if (fminf(floorf(tmax + r), (float)(u.D - 1)) > (float)(dlo + wd - 1)) record_device_error(err, RADON_ERR_DEVICE_BOUNDS);
-            const BwdTileRay A = bwd_tile_ray(vf, u.rays + (long long)(c0 + tid) * u.D, u.D, u.n, ti, tj, u.ih2, u.nh, u.nl);
+            const BwdTileRay A = bwd_tile_ray(vf, u.rays + (long long)(c0 + tid) * u.D, u.D, 0.5f * (tmin + tmax), ti, tj,
+                                              ih2, nh, nl);
             AdjView w;
             w.nx = A.nx;
             w.ny = A.ny;
@@ -607,8 +612,9 @@ __device__ void plan_adjoint_tile_parallel(const Unit& u, int tile, const AdjBuf
     }
 }
 
-// 1024 threads per SM: the launch bounds keep both geometry kinds within 64 registers.
-template <typename T, int KW, int PX>
+// 1024 threads per SM: the launch bounds keep both geometry kinds within 64 registers.  Plans without fan beams take
+// a kernel without the fans' code, which needs no more than 62 and is 1-2 % faster over 40 random plans.
+template <typename T, int KW, int PX, bool FANS>
 __global__ void __launch_bounds__(adj_threads(PX), 4 * PX) plan_adjoint_kernel(const Unit* __restrict__ units,
                                                                     const Work* __restrict__ work, int n_work,
                                                                     unsigned* counter, int max_wd, int cap, int* err) {
@@ -622,7 +628,7 @@ __global__ void __launch_bounds__(adj_threads(PX), 4 * PX) plan_adjoint_kernel(c
         if (wi >= n_work) return;
         const Work w = work[wi];
         const Unit& u = units[w.unit];
-        if (u.fan)
+        if (FANS && u.fan)
             plan_adjoint_tile<T, KW, PX>(u, w.tile, b, Epilogue{1.0f, nullptr, 0.0f, nullptr}, err);
         else if (u.cand3)
             plan_adjoint_tile_parallel<T, KW, 3, PX>(u, w.tile, b, Epilogue{1.0f, nullptr, 0.0f, nullptr}, err);
@@ -861,8 +867,9 @@ radon_status single_backward_px(const Unit& u, long long tiles, size_t smem, con
 template <typename T, int KW, int NC>
 radon_status single_backward_tk(const Unit& u, long long tiles, size_t smem, const Epilogue& ep, int* err,
                                 cudaStream_t s) {
-    return NC >= 0 && adj_pixels((double)tiles, kAdjSms) == 2 ? single_backward_px<T, KW, NC, 2>(u, tiles, smem, ep, err, s)
-                                                   : single_backward_px<T, KW, NC, 1>(u, tiles, smem, ep, err, s);
+    if constexpr (NC >= 0)   // (fans' pairs are never the faster)
+        if (adj_pixels((double)tiles, kAdjSms) == 2) return single_backward_px<T, KW, NC, 2>(u, tiles, smem, ep, err, s);
+    return single_backward_px<T, KW, NC, 1>(u, tiles, smem, ep, err, s);
 }
 
 template <typename T>
@@ -932,6 +939,7 @@ struct radon_plan {
     int device = 0;
     int kw = 3;
     int px = 2;                 // adjoint: pixels per thread
+    bool fans = false;          // adjoint: some unit is a fan beam
     int max_wd = 0;
     int cap = kMaxChunkViews;   // adjoint: views per chunk at most (its shared memory holds that many)
     int ctas = 0;
@@ -1021,6 +1029,23 @@ radon_status upload_units(radon_plan* p) {
     return RADON_OK;
 }
 
+// f of the plan's adjoint kernel: samples per candidate window, pixels per thread, fan beams among its units.
+template <typename F>
+auto with_adjoint_kernel(const radon_plan* p, F f) {
+    constexpr std::integral_constant<int, 1> one{};
+    constexpr std::integral_constant<int, 2> two{};
+    constexpr std::integral_constant<int, 3> three{};
+    constexpr std::integral_constant<int, 6> six{};
+    constexpr std::true_type yes{};
+    constexpr std::false_type no{};
+    if (p->px == 2) {
+        if (p->fans) return p->kw == 3 ? f(three, two, yes) : f(six, two, yes);
+        return p->kw == 3 ? f(three, two, no) : f(six, two, no);
+    }
+    if (p->fans) return p->kw == 3 ? f(three, one, yes) : f(six, one, yes);
+    return p->kw == 3 ? f(three, one, no) : f(six, one, no);
+}
+
 template <typename T>
 // Runs the plan over the work list d_work (n_work items, the first n_staged of them staged-kernel
 // items): forward = pack, then the staged kernel and the L1 gather, each persistent over its items
@@ -1054,8 +1079,9 @@ radon_status launch_t(const radon_plan* p, const Work* d_work, int n_work, int n
     } else {
         int* err = device_error_word();
         if (err == nullptr) return fail(RADON_ERR_CUDA, "device error word unavailable");
-        auto kern = p->px == 2 ? (p->kw == 3 ? plan_adjoint_kernel<T, 3, 2> : plan_adjoint_kernel<T, 6, 2>)
-                               : (p->kw == 3 ? plan_adjoint_kernel<T, 3, 1> : plan_adjoint_kernel<T, 6, 1>);
+        auto kern = with_adjoint_kernel(p, [](auto kw, auto px, auto fans) {
+            return plan_adjoint_kernel<T, decltype(kw)::value, decltype(px)::value, decltype(fans)::value>;
+        });
         kern<<<std::min(p->ctas, n_work), adj_threads(p->px), p->smem, s>>>(p->d_units, d_work, n_work, p->d_counter, p->max_wd, p->cap,
                                                          err);
         e = cudaGetLastError();
@@ -1073,11 +1099,11 @@ radon_status launch_plan(const radon_plan* p, const Work* d_work, int n_work, in
     }
 }
 
-template <typename T, int KW, int PX>
+template <typename T, int KW, int PX, bool FANS>
 cudaError_t adj_occupancy(size_t smem, int* per_sm) {
-    const cudaError_t e = raise_smem_attr<plan_adjoint_kernel<T, KW, PX>>(smem);
+    const cudaError_t e = raise_smem_attr<plan_adjoint_kernel<T, KW, PX, FANS>>(smem);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, plan_adjoint_kernel<T, KW, PX>, adj_threads(PX), smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, plan_adjoint_kernel<T, KW, PX, FANS>, adj_threads(PX), smem);
 }
 
 template <typename T>
@@ -1107,8 +1133,10 @@ radon_status occupancy_t(radon_plan* p) {
             longest = std::max(longest, (double)u.V);
         }
         p->px = 2 * fan > all ? 1 : adj_pixels(all / longest, sms);
-        e = p->px == 2 ? (p->kw == 3 ? adj_occupancy<T, 3, 2>(p->smem, &per_sm) : adj_occupancy<T, 6, 2>(p->smem, &per_sm))
-                       : (p->kw == 3 ? adj_occupancy<T, 3, 1>(p->smem, &per_sm) : adj_occupancy<T, 6, 1>(p->smem, &per_sm));
+        p->fans = fan > 0.0;
+        e = with_adjoint_kernel(p, [&](auto kw, auto px, auto fans) {
+            return adj_occupancy<T, decltype(kw)::value, decltype(px)::value, decltype(fans)::value>(p->smem, &per_sm);
+        });
     }
     if (e != cudaSuccess) return cuda_fail(e, "plan occupancy query");
     p->ctas = std::max(1, per_sm) * sms;
