@@ -57,8 +57,12 @@ int backward_packed_images_per_cta(const radon_geometry* g, int batch, radon_dty
     if (g->fan && bwdp_table_serves(g, 16) && dt != RADON_F32) return 16;
     // A 32-image CTA costs about 1.56x a 16-image one (1.36-1.51x on parallel 512^2 with 512 views, 1.6x
     // on 360-view fans with 1024 detectors): take it when its groups cost less and its staging fits one CTA's
-    // shared memory.
+    // shared memory -- but not on few tiles, where a CTA's four gathering warps wait for their own loads and
+    // groups of 16 make twice the warps (us, 32 -> 16, 32 FP16 images, 100 views: fan 100^2 95 -> 75, parallel
+    // 64 -> 51; at 150^2, 200 CTAs of 16, 94 -> 92 and 63 -> 66).
     const long long g32 = (batch + 31) / 32, g16 = (batch + 15) / 16;
+    const long long side = (g->n + kBwdTile - 1) / kBwdTile;
+    if (side * side * g16 <= 152) return 16;
     if (25 * g32 < 16 * g16 && smem_32(g, dt) <= 227 * 1024) return 32;
     return 16;
 }
