@@ -156,6 +156,19 @@ cudaError_t launch_packed_ng(const CUtensorMap& mr, const CUtensorMap& mc, const
         if (e != cudaSuccess) return e;
         attr_bytes = smem;
     }
+    if constexpr (ROWS && NG < 4) {   // beside the launch of four groups before it
+        cudaLaunchAttribute beside;
+        beside.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        beside.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t c = {};
+        c.gridDim = grid;
+        c.blockDim = dim3(kFwdThreads);
+        c.dynamicSmemBytes = smem;
+        c.stream = s;
+        c.attrs = &beside;
+        c.numAttrs = 1;
+        return cudaLaunchKernelEx(&c, kern, mr, mc, a);
+    }
     kern<<<grid, kFwdThreads, smem, s>>>(mr, mc, a);
     return cudaGetLastError();
 }
@@ -356,9 +369,11 @@ radon_status launch_forward_packed(radon_geometry* g, const void* packed, void* 
     };
     // One or two groups past whole CTAs of four run by themselves, row by row like the others with the same slabs, so
     // that equal images of a batch have equal projections; and with their code out of the kernel of four
-    // groups it keeps its registers (us, one launch that takes them sample by sample -> two: 32 x 512^2, 512
-    // views, no tail, FP16 1387 -> 1352, BF16 1283 -> 1206; 34 FP16 images 1988 -> 1941, 41 2182 -> 2187; FP32 38
-    // x 256^2, 256 views 339 -> 324).  Two groups take two CTAs per SM (96 registers; at three 72 spill: 41 2220).
+    // groups it keeps its registers.  They start as the last CTAs of four do (their inputs were packed before
+    // that launch, their outputs are other images) and fill the SMs that those leave.  (us, one launch that
+    // takes them sample by sample -> two one after the other -> two so, FP16: 34 x 512^2, 512 views 1993 ->
+    // 1941 -> 1782; 40 x 256^2, 202 views 283 -> 333 -> 274; 100 x 128^2, 162 views 148 -> 186 -> 152; no tail,
+    // 32 x 512^2, 512 views 1387 -> 1345, BF16 1279 -> 1203.)
     const int tail = sh.NG == 4 && groups % 4 <= 2 ? groups % 4 : 0;
     radon_status done = launch(0, groups - tail, sh.NG, sh.stages, sh.smem, sh.NG == 4);
     if (done == RADON_OK && tail > 0) {

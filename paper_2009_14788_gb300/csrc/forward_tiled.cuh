@@ -790,6 +790,8 @@ __global__ void __launch_bounds__(kFwdThreads, ROWS && NG >= 2 ? 2 : 3) forward_
     }
     fence_mbar_init();
     __syncthreads();
+    // the groups left over may start once every CTA of this launch has
+    if constexpr (NG == 4) grid_launch_dependents();
 
     if (warp == kFwdConsumerWarps) {
         const int lane = tid & 31;
@@ -831,6 +833,9 @@ __global__ void __launch_bounds__(kFwdThreads, ROWS && NG >= 2 ? 2 : 3) forward_
     else   // one group (or a pair whose second group lies past the batch: its plane is never read)
         fwd_consume<T, MODE, 1, LN, ROWS>(a, cls, v0, cnt, d0, b0, full, empty, band_xc0, band_bad, abort_flag,
                                           comp_base, comp_stride, a.wbox, slab_rng);
+    // ... and their launch ends after the one that they started beside: what follows on the stream waits for both
+    if constexpr (ROWS && NG < 4)
+        if (blockIdx.x == 0) grid_wait_prerequisites();
 }
 
 }  // namespace radon

@@ -155,4 +155,10 @@ __device__ __forceinline__ void sts1(uint32_t a, float v) {
     asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
 }
 
+// Programmatic dependent launch: lets the next launch, made with the attribute for it, start once every CTA of this
+// grid has called this or ended; and waits until the grids that this one was started beside are complete
+// and their writes visible (nothing to wait for without the attribute).
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 }  // namespace radon
