@@ -180,8 +180,8 @@ __device__ __forceinline__ float bwdp_weight(float px, float py, float s, const 
 //   (l - l0) n + s step - p + A          sample s of window ray l relative to the pixel
 // A candidate ray then costs a pixel two additions and its samples' tents instead of a record's two shared
 // loads, its first sample and its offset from the pixel, and no ray rows are copied or re-based (us, ray
-// records -> one ray per view, FP32, 512 views of 512^2: 8 images 898 -> 675, 16 images 1056 -> 854, 32
-// images 1581 -> 1286; 4 x 64^2, 64 views: 42 -> 30).
+// records -> one ray per view, FP32, 512 views of 512^2: 8 images 898 -> 667, 16 images 1056 -> 859, 32
+// images 1581 -> 1266; 4 x 64^2, 64 views: 42 -> 26).
 struct BwdPPar {
     float nx, ny, t0, c;
     float Ax, Ay, sx, sy;

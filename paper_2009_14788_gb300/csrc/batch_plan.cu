@@ -655,9 +655,10 @@ size_t adj_smem_bytes(int max_wd, int cap) {
 constexpr int kAdjSms = 152;
 
 // Pixels per thread of a parallel-beam adjoint launch with the work of `tiles` tiles as long as its longest: a
-// pair is less work, single pixels twice the warps, which a launch of few tiles wants (us, single -> pair:
-// one image of 64^2 36 -> 42, 256^2 48 -> 48, 448^2, 5.2 tiles per SM, 120 -> 115, 512^2 138 -> 132; plans
-// of 0.7 tiles per SM 98 -> 121, 3.9 289 -> 314, 4.5 186 -> 173, 8.9 471 -> 456, 12.7 260 -> 229).  Fans' pairs
+// pair is less work, single pixels twice the warps, which a launch of few tiles wants (us, single -> pair: one
+// image, 200 views, of 64^2 30 -> 37, 256^2 42 -> 45, 384^2, 3.8 tiles per SM, 77 -> 79, 448^2, 5.2, 111 -> 109,
+// 512^2 128 -> 125, 700^2 229 -> 220; plans of 0.8 tiles per SM 39 -> 49, 3.9 285 -> 317, 6.7 199 -> 194, 10.5
+// 345 -> 320, two of 512^2, 13.5, 538 -> 479).  Fans' pairs
 // share little and are never the faster (64^2 112 -> 176, 576^2 494 -> 515).
 int adj_pixels(double tiles, int sms) { return tiles >= 4.5 * sms ? 2 : 1; }
 
