@@ -39,13 +39,15 @@ constexpr int kBwdPMaxStages = 4;        // ring depth limit (mbarrier slots in 
 // and window row loaded from shared memory serves both pixels' accumulators.  For 32-image groups the pair
 // fills 127 registers at three CTAs per SM (two pixels x 32 sums); one pixel per thread, four CTAs' worth
 // of warps, read every row twice as often: parallel 32 x 512^2, 512 views, FP16 1.92 -> 1.70 ms, and
-// 1.54 ms with the records' second half cut to the one word that cannot be recomputed.
-template <int BG>
+// 1.54 ms with the records' second half cut to the one word that cannot be recomputed.  The interpolating
+// backprojector's two taps per pixel share nothing with the neighbour's: its 32-image groups keep one pixel per
+// thread (32 x 256^2, 100 views, FP16: fan 88 us in pairs, 79 so; parallel 84, 74).
+template <int BG, bool INTERP>
 struct BwdPShape {
-    static constexpr int PX = 2;
+    static constexpr int PX = INTERP && BG == 32 ? 1 : 2;
     static constexpr int kConsumers = kBwdThreads / PX;
     static constexpr int kThreads = kConsumers + 32;
-    static constexpr int kCtasPerSm = BG <= 16 ? 4 : 3;   // resident CTAs the launch bounds ask for
+    static constexpr int kCtasPerSm = BG <= 16 ? 4 : PX == 2 ? 3 : 2;   // resident CTAs the launch bounds ask for
 };
 constexpr size_t kBwdPHeader = 1024;     // barriers, flags, windows and view maps of the ring
 
@@ -291,7 +293,7 @@ __device__ __forceinline__ void bwdp_widen8<__nv_bfloat16>(const uint4 u, float4
 // view in which some pair of the tile overflows the table (the table's per-view flags).  The producer
 // prefetches the table's rows for the chunk that will next reuse its ring slot into L2.
 template <typename T, int BG, int KW, bool TAB, bool PAR>
-__global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasPerSm)
+__global__ void __launch_bounds__(BwdPShape<BG, KW == 0>::kThreads, BwdPShape<BG, KW == 0>::kCtasPerSm)
     backward_packed_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap rmap,
                            const BwdPArgs a) {
     static_assert(!TAB || (KW > 0 && BG <= 16 && (!PAR || (BG == 16 && KW == 6))),
@@ -301,8 +303,8 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
     using L = BwdPLayout<T, BG>;
     constexpr int NQ = BG / 4;
     constexpr int PITCH = L::kPitch;
-    constexpr int PX = BwdPShape<BG>::PX;
-    constexpr int NC = BwdPShape<BG>::kConsumers;
+    constexpr int PX = BwdPShape<BG, KW == 0>::PX;
+    constexpr int NC = BwdPShape<BG, KW == 0>::kConsumers;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127);
     uint64_t* tma_bar = reinterpret_cast<uint64_t*>(smem);        // [stages]: a slot's copies landed
@@ -437,9 +439,16 @@ __global__ void __launch_bounds__(BwdPShape<BG>::kThreads, BwdPShape<BG>::kCtasP
     // each warp takes an 8 x 8 block of the tile, lanes on a 4 x 8 grid of vertical pixel pairs: a block's
     // detector footprints overlap more than those of a strip, so the gather's shared loads touch fewer
     // distinct addresses.  A 16-byte shared load is served eight lanes at a time, so each group of eight
-    // lanes covers a compact block of 2 x 4 pairs, whose detector span stays within the eight bank groups
+    // lanes covers a compact block of 2 x 4 pairs, whose detector span stays within the eight bank groups (of
+    // 4 x 2 pixels in blocks of 4 x 8 where a thread owns one)
     int pi0, pj;
-    bwdp_pair_of(tid, &pi0, &pj);
+    if constexpr (PX == 2) {
+        bwdp_pair_of(tid, &pi0, &pj);
+    } else {
+        const int grp = (tid & 31) >> 3, e8 = tid & 7;
+        pi0 = (tid >> 6) * 4 + (e8 >> 1);
+        pj = ((tid >> 5) & 1) * 8 + grp * 2 + (e8 & 1);
+    }
     const float px = (float)pj, py0 = (float)pi0;
     const float gx = (float)(tj + pj), gy0 = (float)(ti + pi0);
     float acc[PX][BG];
@@ -854,8 +863,9 @@ __global__ void __launch_bounds__(kBwdTabPairs) bwdp_table_kernel(const RayT* __
 // bounds' CTAs resident per SM (228 KB of shared memory, 1 KB reserved per CTA), else two stages;
 // returns the dynamic shared memory.
 template <typename T, int BG>
-inline size_t bwdp_plan(int wd, bool rays, int* stages) {
-    const size_t budget = (size_t)228 * 1024 / BwdPShape<BG>::kCtasPerSm - 1024;
+inline size_t bwdp_plan(int wd, bool rays, int* stages, bool interpolating = false) {
+    const int ctas = interpolating ? BwdPShape<BG, true>::kCtasPerSm : BwdPShape<BG, false>::kCtasPerSm;
+    const size_t budget = (size_t)228 * 1024 / ctas - 1024;
     int S = kBwdPMaxStages;
     while (S > 2 && bwdp_smem<T, BG>(wd, S, rays).total > budget) --S;
     *stages = S;
@@ -883,7 +893,7 @@ cudaError_t bwdp_launch(const CUtensorMap& map, const CUtensorMap& rmap, const B
         if (e != cudaSuccess) return e;
         attr_bytes = smem;
     }
-    kern<<<grid, BwdPShape<BG>::kThreads, smem, s>>>(map, rmap, a);
+    kern<<<grid, BwdPShape<BG, KW == 0>::kThreads, smem, s>>>(map, rmap, a);
     return cudaGetLastError();
 }
 
@@ -907,7 +917,7 @@ radon_status launch_backward_packed_t(const radon_geometry* g, const void* packe
     const bool tab = kw > 0 && bwdp_table_serves(g, BG) && g->tab_kw == kw && g->tab_wd == wd;
     int stages = 2;
     // ray rows are staged for fans (with a table too, for the pairs it marks as overflowing)
-    const size_t smem = bwdp_plan<T, BG>(wd, kw > 0 && !par, &stages);
+    const size_t smem = bwdp_plan<T, BG>(wd, kw > 0 && !par, &stages, kw == 0);
     if (smem > 227 * 1024) {
         *why = "shared memory budget exceeded";
         return RADON_ERR_UNSUPPORTED;

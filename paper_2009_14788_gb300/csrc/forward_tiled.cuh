@@ -750,7 +750,8 @@ __global__ void __launch_bounds__(kFwdThreads, 3) forward_tiled_kernel(const __g
 // Packed variant: the image batch was packed once into 16-byte texels (rows / cols copies, see
 // pack.cu), so the producer warp only bounds each band and copies it with one 4-D TMA load straight
 // into the compute buffer it will become (row pitch = band width); no staging, no repack.
-// ROWS: rays go row by row where they can (four groups, and the one or two left over from a launch of four).
+// ROWS: rays go row by row where they can (four groups, and the one or two left over from a launch of four).  Two
+// CTAs per SM leave them 96 registers; four 16-bit groups spill 24 bytes, FP32 ones 4.
 template <typename T, int MODE, int NG, int LN, bool ROWS>
 __global__ void __launch_bounds__(kFwdThreads, ROWS && NG >= 2 ? 2 : 3) forward_packed_kernel(const __grid_constant__ CUtensorMap map_rows,
                                                                        const __grid_constant__ CUtensorMap map_cols,
