@@ -219,27 +219,35 @@ radon_status packed_forward_shape(radon_geometry* g, radon_dtype dt, int batch, 
     // texels (4 images each) measured slower paired.  Rows per slab: 16 for one group; 14 for two
     // (2 CTAs/SM), 8 with FP16 weights (3 CTAs/SM), the fastest of 8-16 rows measured.  A default pair
     // whose buffers would not fit falls back to one group.
-    // Four groups, row by row, where the batch fills most of one more CTA: 16-bit batches of more than
-    // 24 images (parallel 32 x 512^2, 512 views: FP16 1.78 -> 1.35 ms, BF16 1.55 -> 1.20; three groups cost
-    // about what a pair and a single do) and FP32 batches of more than 16 (2.33 -> 1.56 ms; 32 x 256^2, 256
-    // views 376 -> 242 us; smaller FP32 batches keep the one group that the query reports for them), in
-    // the highest slab of 8, 6 or 4 rows that leaves two CTAs per SM (with the left-over groups still in the
-    // kernel, FP16: 8 rows 1.45 ms, 6 1.48, 4 1.56; 10 rows at one CTA 1.88).  FP16 weights keep two groups.  Not where the CTAs of four groups would not fill
-    // two per SM (us, default -> four groups, FP16: 32 x 256^2, 128 views, 204 CTAs 177 -> 194; 192 views, 300
-    // CTAs 242 -> 239; 256 views, 396 CTAs 284 -> 246), nor, since a CTA costs the same with empty groups and
-    // thin slabs repeat the rows between them, where groups are empty and the slab is low: FP32, against one
-    // group per CTA, needs 6 rows (32 x 512^2, 100 views, 4 rows: 682 -> 891; 32 x 256^2, 128 views, 6 rows:
-    // 219 -> 178), either type two more with two groups empty (FP32 24 x 256^2, 256 views, 8 rows: 289 -> 239;
-    // 24 x 266^2 fan, 586 views, 6 rows: 570 -> 640) and FP32 never runs with three (20 x 512^2, 150 views:
-    // 579 -> 958).  (One or two groups past whole CTAs now run beside them and cost less: 24 x 256^2, 256 views,
-    // 201.)
+    // Four groups, row by row, where the batch fills most of one more CTA: 16-bit batches of more than 24 images
+    // (parallel 32 x 512^2, 512 views: FP16 1.78 -> 1.35 ms, BF16 1.55 -> 1.20; three groups cost about what a pair
+    // and a single do) and FP32 batches of more than 16 (2.33 -> 1.56 ms; 32 x 256^2, 256 views 376 -> 242 us; smaller
+    // FP32 batches keep the one group that the query reports for them), in the highest slab of 8, 6 or 4 rows that
+    // leaves two CTAs per SM (with the left-over groups still in the kernel, FP16: 8 rows 1.45 ms, 6 1.48, 4 1.56; 10
+    // rows at one CTA 1.88).  FP16 weights keep two groups.  Not where the CTAs of four groups would not fill two per
+    // SM (us, default -> four groups, FP16: 32 x 256^2, 128 views, 204 CTAs 177 -> 194; 192 views, 300 CTAs 242 ->
+    // 239; 256 views, 396 CTAs 284 -> 246), nor, since a CTA costs the same with empty groups and thin slabs repeat
+    // the rows between them, where groups are empty and the slab is low: FP32, against one group per CTA, needs 6 rows
+    // (32 x 512^2, 100 views, 4 rows: 682 -> 891; 32 x 256^2, 128 views, 6 rows: 219 -> 178), either type two more
+    // with two groups empty (FP32 24 x 256^2, 256 views, 8 rows: 289 -> 239; 24 x 266^2 fan, 586 views, 6 rows: 570 ->
+    // 640) and FP32 never runs with three (20 x 512^2, 150 views: 579 -> 958).
+    // Nor where too few of the samples lie on rays that go by rows: sample by sample four groups only leave fewer CTAs
+    // (steps other than one pixel; us, default -> four groups at a share of 0 | 0.4 | 0.6 | 0.75 | 0.85: 32 x 512^2,
+    // 300 views, FP32 2104 -> 2306 | 1858 -> 1608 | 1759 -> 1383; 25 x 215^2, 219 views, 314 -> 418 | 279 -> 311 | 266
+    // -> 272 | 253 -> 237; 32 x 256^2, 256 views, FP16 438 -> 463 | 382 -> 469 | 357 -> 400 | 337 -> 337, and 512^2
+    // 1686 -> 1753 | 1472 -> 1315 | 1382 -> 1151; with steps above one, where the rays nearest the rows' normal fall
+    // out, 273 -> 322 and 1043 -> 1040 at 0.75; where some do not, twice the CTAs are needed to even out those that
+    // take longer: at 0.85, 396 CTAs, 320 -> 357).  (One or two groups past whole CTAs now run beside them and cost
+    // less: 24 x 256^2, 256 views, 201.)
     const int groups = (batch + BG - 1) / BG;
     const int empty = groups < 12 ? (4 - groups % 4) % 4 : 0;   // (of many, a few cost little)
     const int min_rows = 4 + (esz == 4 ? 2 : 0) + (empty >= 2 ? 2 : 0);
     const long long ctas4 = (long long)g->group_count[G >= 8 ? 3 : G >= 4 ? 2 : G >= 2 ? 1 : 0] * ((g->D + Dt - 1) / Dt) *
                             ((groups + 3) / 4);
     const int fixed_rows = cfg ? cfg->rows_per_slab : 0;
-    const bool four = !f16w && batch > (esz == 2 ? 24 : 16) && !(esz == 4 && empty == 3) && ctas4 >= kFwdFourMinCtas &&
+    const double min_share = esz == 4 ? 0.55 : g->h > 1.0 ? 0.9 : 0.7;
+    const bool four = !f16w && g->row_share >= min_share && batch > (esz == 2 ? 24 : 16) && !(esz == 4 && empty == 3) &&
+                      ctas4 >= kFwdFourMinCtas * (g->row_share < 0.98 ? 2 : 1) &&
                       (fixed_rows == 0 || fixed_rows >= min_rows);
     int NG = lanes == 2 ? 1
              : ipc != 0 ? (ipc == 2 * BG ? 2 : 1)

@@ -353,8 +353,6 @@ __device__ void fwd_repack(const FwdTiledArgs& a, int cls, int yoff, const unsig
 // per row and 0.9 rows per sample instead of four texels per sample.  With tent(x - c) = sat(x - c + 1) -
 // sat(x - c), the weights are differences of P_j = sum_k tent(y_k - r) sat(x_k - c0 - j): three samples
 // and three columns take nine saturating additions and nine products.
-constexpr float kRowMinStep = 0.668f;   // rows between samples from which three samples span a row's two
-
 template <typename T, int MODE>
 struct FwdRow {
     float dX, dY, rdY, sX, sY;   // step, 1 / dY, base sample
@@ -447,7 +445,7 @@ __device__ void fwd_consume(const FwdTiledArgs& a, int cls, int v0, int cnt, int
     // the steepest of such a fan; with shorter steps the rays nearest the rows' normal, down to 0.668 rows a
     // step.  Other rays, and launches of one or two groups, over which a row's weights do not pay (8 BF16
     // images 126 -> 151 us, 16 FP16 images 1.39 -> 1.38 ms), go sample by sample.
-    const bool by_row = ROWS && nk > 0 && dY >= kRowMinStep && dY <= 1.0001f && fabsf(dX) <= 0.75f;
+    const bool by_row = ROWS && nk > 0 && forward_by_rows(dX, dY);
     const float rdY = by_row ? 1.0f / dY : 0.0f;
     int r_lo = 0, r_hi = -1;   // texel rows the ray's samples reach
     if (by_row) {

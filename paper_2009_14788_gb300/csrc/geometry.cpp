@@ -118,7 +118,7 @@ radon_status build_geometry(radon_geometry* g) {
     g->h_ray.assign((size_t)V * D, RayT{0, 0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f});
     g->h_nk.assign((size_t)V * D, 0);
     g->h_view.assign((size_t)V, ViewF{});
-    int64_t total = 0;
+    int64_t total = 0, by_rows = 0;
     int max_nk = 0;
     for (int v = 0; v < V; ++v) {
         const double th = g->angles[v];
@@ -198,10 +198,13 @@ radon_status build_geometry(radon_geometry* g) {
             rt.dyl = (float)(sy - hy);
             g->h_nk[idx] = nk;
             total += nk;
+            const float fx = rt.dxh + rt.dxl, fy = rt.dyh + rt.dyl;
+            if (forward_by_rows(major == 0 ? fx : fy, major == 0 ? fy : fx)) by_rows += nk;
             if (nk > max_nk) max_nk = nk;
         }
     }
     g->samples = total;
+    g->row_share = total > 0 ? (double)by_rows / (double)total : 0.0;
     g->max_nk = max_nk;
     g->bwd_window = backward_window_width(g, 16);
     // The tiled forward gives each 8-lane phase of its 16-byte shared loads two neighbouring views x

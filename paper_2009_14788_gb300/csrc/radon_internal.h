@@ -59,6 +59,16 @@ struct Int2 {
     int x, y;
 };
 
+// Whether the forward's row mode takes a ray of the compute-frame step (dX, dY): at most three of its samples reach a
+// texel row, over at most four columns.
+constexpr float kRowMinStep = 0.668f;   // rows between samples from which three samples span a row's two
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline bool forward_by_rows(float dX, float dY) {
+    return dY >= kRowMinStep && dY <= 1.0001f && (dX < 0.0f ? -dX : dX) <= 0.75f;
+}
+
 }  // namespace radon
 
 struct radon_geometry {
@@ -68,6 +78,7 @@ struct radon_geometry {
     int64_t samples = 0;
     int max_nk = 0;
     int bwd_window = 0;               // widest detector window of a 16x16 tile (tiled adjoint)
+    double row_share = 0.0;           // share of the samples on rays that the forward can take row by row
     int fwd_pair_views = 0;           // tiled forward: two views x four detectors per load phase
     std::vector<radon::Int2> h_groups;  // view groups for G = 1, 2, 4, 8 (concatenated)
     int group_offset[4] = {0, 0, 0, 0};
