@@ -244,11 +244,11 @@ RADON_API size_t radon_forward_workspace_size(const radon_geometry* geometry, ra
  * sample's position, floor and weight evaluation (16 / 8), or four that share each texel row's weights (32
  * / 16).  By default 16-bit batches of more than 8 images take two groups and of more than 24 four (FP32
  * weights), FP32 batches of more than 16 images four and smaller ones one -- where the bands leave two such
- * CTAs room on an SM, the batch fills their groups and the CTAs fill the GPU, else fewer groups; `config`'s
- * images_per_cta chooses where it holds one or two groups' images.  A batch of one group on few CTAs takes
- * two threads per ray over four views.  Where no shape with one thread per ray fits a TMA box (sparse views
- * with a detector wider than the image) and `config` fixes no views per CTA, two threads share each ray (half
- * the detectors per CTA, one texel group).  Equal images of one batch have the same projections bit for bit;
+ * CTAs room on an SM, the batch fills their groups, the CTAs fill the GPU and the steps are near one pixel, else
+ * fewer groups; `config`'s images_per_cta chooses where it holds one or two groups' images.  A batch of one
+ * group on few CTAs takes two threads per ray over four views.  Where no shape with one thread per ray fits a
+ * TMA box (sparse views with a detector wider than the image) and `config` fixes no views per CTA, two threads
+ * share each ray (half the detectors per CTA, one texel group).  Equal images of one batch have the same projections bit for bit;
  * between batches of different sizes, which may take other shapes, the order of a ray's sum and so its last
  * bits can differ.  *images = 0 when another kernel serves the call (one image under AUTO, the PLAIN
  * algorithm, a geometry no packed shape takes).  Host only (host-only geometries are answered too); no
