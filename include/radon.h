@@ -274,8 +274,9 @@ RADON_API radon_status radon_forward_ws(const radon_geometry* geometry, const vo
  * holding the group's images in the storage type (bg 16-bit values, or bg FP32 values and four
  * padding words).  Groups of bg = 8 images for batches of at most 8, 16 up to 16; above that 16 for
  * 16-bit storage when a fan geometry holds an adjoint weight table, else 32 where whole groups of 32
- * cost less than groups of 16 (a 32-image CTA costs ~1.56x a 16-image one) and their staging fits
- * one CTA's shared memory, else 16.  Returns 0 for an invalid geometry, dtype or batch.
+ * cost less than groups of 16 (a 32-image CTA costs ~1.56x a 16-image one), their staging fits one
+ * CTA's shared memory and the 16 x 16 tiles of groups of 16 are more than 152, else 16.  Returns 0 for an
+ * invalid geometry, dtype or batch.
  */
 RADON_API size_t radon_backward_workspace_size(const radon_geometry* geometry, radon_dtype dtype, int batch);
 
